@@ -68,7 +68,8 @@ typedef enum {
 /* Kernel structure of one step. */
 typedef enum {
   SWE_KERNEL_AUTO = 0,  /* SWE_KERNEL_TILED; SWE_KERNEL_EDGE for a single mesh in
-                           SWE_ORDER_RCM, whose tiles would be thin strips */
+                           SWE_ORDER_RCM, whose tiles would be thin strips; small meshes
+                           stay on chip for many steps (see swe_params.tile) */
   SWE_KERNEL_EDGE = 1,  /* two launches: per-edge fluxes to HBM, then a per-cell gather
                            and update (the paper's two parallel loops, Sec. 2.3) */
   SWE_KERNEL_TILED = 2  /* one launch: each block stages a tile of cells in shared
@@ -232,7 +233,8 @@ swe_status swe_step(swe_state* state, double* dt_used);
 /* Queues n_steps steps of swe_step (Eq. 4, each with its CFL dt, Sec. 2.2)
  * without an end time and returns without synchronising (device errors are
  * reported by the next synchronising call). Steps are replayed from
- * captured CUDA graphs; the host reads nothing back between them (Sec. 2.3:
+ * captured CUDA graphs (meshes that stay on chip: one launch of up to 4,096
+ * steps); the host reads nothing back between them (Sec. 2.3:
  * no transfer during the time loop). n_steps = 0 takes no step and only
  * captures (and uploads) the step graph if the state has none yet, so that
  * the steps of a later call are replayed from its first one. */

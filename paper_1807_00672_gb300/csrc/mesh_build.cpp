@@ -48,18 +48,26 @@ std::vector<int32_t> morton_order(const double* xy, int64_t V, const int32_t* tr
   double span = std::max(x1 - x0, y1 - y0);
   if (!(span > 0.0)) span = 1.0;
   const double q = 4194303.0;  // 22 bits per axis
-  std::vector<uint64_t> key(T);
+  // Stable radix sort of (key, cell) by the 44 key bits, 11 at a time.
+  struct Item { uint64_t key; int64_t cell; };
+  std::vector<Item> a(T), b(T);
   for (int64_t i = 0; i < T; ++i) {
-    int32_t a = tri[3 * i], b = tri[3 * i + 1], c = tri[3 * i + 2];
-    double cx = (xy[2 * a] + xy[2 * b] + xy[2 * c]) / 3.0;
-    double cy = (xy[2 * a + 1] + xy[2 * b + 1] + xy[2 * c + 1]) / 3.0;
+    int32_t p = tri[3 * i], r = tri[3 * i + 1], c = tri[3 * i + 2];
+    double cx = (xy[2 * p] + xy[2 * r] + xy[2 * c]) / 3.0;
+    double cy = (xy[2 * p + 1] + xy[2 * r + 1] + xy[2 * c + 1]) / 3.0;
     uint64_t ix = (uint64_t)std::min(q, std::max(0.0, (cx - x0) / span * q));
     uint64_t iy = (uint64_t)std::min(q, std::max(0.0, (cy - y0) / span * q));
-    key[i] = spread_bits(ix) | (spread_bits(iy) << 1);
+    a[i] = {spread_bits(ix) | (spread_bits(iy) << 1), i};
+  }
+  for (int shift = 0; shift < 44; shift += 11) {
+    std::vector<int64_t> at(2049, 0);
+    for (const Item& x : a) at[((x.key >> shift) & 2047) + 1]++;
+    for (int d = 0; d < 2048; ++d) at[d + 1] += at[d];
+    for (const Item& x : a) b[at[(x.key >> shift) & 2047]++] = x;
+    a.swap(b);
   }
   std::vector<int32_t> order(T);
-  std::iota(order.begin(), order.end(), 0);
-  std::stable_sort(order.begin(), order.end(), [&](int32_t p, int32_t r) { return key[p] < key[r]; });
+  for (int64_t i = 0; i < T; ++i) order[i] = (int32_t)a[i].cell;
   return order;
 }
 
@@ -265,7 +273,8 @@ void bank_order(const std::vector<int32_t>& tA, const std::vector<int32_t>& tB, 
   }
 }
 
-// Applies bank_order to every tile of m (host threads over tiles).
+}  // namespace
+
 void order_records_for_banks(HostMesh& m) {
   const int64_t nt = m.ntiles;
   unsigned nth = std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
@@ -306,10 +315,8 @@ void order_records_for_banks(HostMesh& m) {
   for (std::thread& th : pool) th.join();
 }
 
-}  // namespace
-
 int build_host_mesh(const double* xy, int64_t V, const int32_t* tri_in, int64_t T, int order,
-                    int32_t tile, bool with_edges, HostMesh& m, bool bank) {
+                    int32_t tile, bool with_edges, HostMesh& m, bool bank, bool keep_edges) {
   if (!xy || !tri_in || V <= 0 || T <= 0) return T == 0 ? -2 : -1;
   if (T >= (int64_t)INT32_MAX / 3 || V >= (int64_t)INT32_MAX) return -1;
   m = HostMesh();
@@ -565,7 +572,176 @@ int build_host_mesh(const double* xy, int64_t V, const int32_t* tri_in, int64_t 
     if (m.halo_cap == 0) m.halo_cap = 4;
     if (bank) order_records_for_banks(m);
   }
+  if (keep_edges) {
+    m.edges.cL = std::move(cL);
+    m.edges.cR = std::move(cR);
+    m.edges.of_half = std::move(edge_of_half);
+    m.edges.nx = std::move(gnx);
+    m.edges.ny = std::move(gny);
+    m.edges.len = std::move(glen);
+  }
   return 0;
+}
+
+bool build_resident_parts(const HostMesh& m, const double* xy, const int32_t* tri, bool is_morton,
+                          int32_t nparts, ResidentParts& out) {
+  const int64_t T = m.T;
+  const HostEdges& ed = m.edges;
+  out = ResidentParts();
+  if (nparts < 1 || nparts > T || (int64_t)ed.of_half.size() != 3 * T) return false;
+  // Host threads over the parts (ranges whose thread cannot start run here).
+  const unsigned nth = (unsigned)std::min<int64_t>(
+      std::min(8u, std::max(1u, std::thread::hardware_concurrency())), std::min<int64_t>(nparts, T / 4000 + 1));
+  auto over_parts = [&](auto&& body) {
+    std::vector<std::thread> pool;
+    unsigned started = 0;
+    auto run = [&](unsigned k) {
+      body((int32_t)((int64_t)nparts * k / nth), (int32_t)((int64_t)nparts * (k + 1) / nth));
+    };
+    try {
+      for (; started + 1 < nth; ++started) pool.emplace_back(run, started + 1);
+    } catch (...) {
+    }
+    run(0);
+    for (unsigned k = started + 1; k < nth; ++k) run(k);
+    for (std::thread& th : pool) th.join();
+  };
+  // internal cells in Morton order, and the part of each
+  std::vector<int32_t> ord, part(T), local(T), nshared(nparts, 0);
+  if (!is_morton) {
+    ord = morton_order(xy, m.V, tri, T);
+    for (int64_t r = 0; r < T; ++r) ord[r] = m.iperm[ord[r]];
+  }
+  auto cell_at = [&](int64_t r) { return is_morton ? (int32_t)r : ord[r]; };
+  auto first = [&](int32_t b) { return T * b / nparts; };
+  over_parts([&](int32_t b0, int32_t b1) {
+    for (int32_t b = b0; b < b1; ++b)
+      for (int64_t r = first(b); r < first(b + 1); ++r) part[cell_at(r)] = b;
+  });
+  auto neighbour = [&](int64_t c, int k) -> int64_t {  // internal cell across face k of caller cell c, or -1
+    const int32_t e = ed.of_half[3 * c + k];
+    const int32_t o = ed.cL[e] == c ? ed.cR[e] : ed.cL[e];
+    return o < 0 ? -1 : m.iperm[o];
+  };
+  // each part's cells: those that another part reads, then the others
+  out.cells.resize(T);
+  out.pub.assign(T, -1);
+  out.cell0.resize(nparts + 1);
+  for (int32_t b = 0; b <= nparts; ++b) out.cell0[b] = (int32_t)first(b);
+  over_parts([&](int32_t b0, int32_t b1) {
+    std::vector<int32_t> inner;
+    for (int32_t b = b0; b < b1; ++b) {
+      inner.clear();
+      int64_t at = first(b);
+      for (int64_t r = first(b); r < first(b + 1); ++r) {
+        const int32_t i = cell_at(r);
+        const int64_t c = m.perm[i];
+        bool shared = false;
+        for (int k = 0; k < 3; ++k) {
+          const int64_t o = neighbour(c, k);
+          shared = shared || (o >= 0 && part[o] != b);
+        }
+        if (shared) out.cells[at++] = i;
+        else inner.push_back(i);
+      }
+      nshared[b] = (int32_t)(at - first(b));
+      std::copy(inner.begin(), inner.end(), out.cells.begin() + at);
+      for (int64_t q = first(b); q < first(b + 1); ++q) local[out.cells[q]] = (int32_t)(q - first(b));
+    }
+  });
+  std::vector<int32_t> pub0(nparts + 1, 0);
+  for (int32_t b = 0; b < nparts; ++b) {
+    pub0[b + 1] = pub0[b] + nshared[b];
+    for (int32_t q = 0; q < nshared[b]; ++q) out.pub[first(b) + q] = pub0[b] + q;
+    out.cell_cap = std::max<int32_t>(out.cell_cap, (int32_t)(first(b + 1) - first(b)));
+  }
+  out.npub = pub0[nparts];
+
+  // each part's records (own cells, walls, then halo cells: the first two
+  // run while the words of the halo cells arrive) and halo list
+  struct Rec { uint32_t side; int32_t e; };
+  struct Part {
+    std::vector<Rec> recs;
+    std::vector<int32_t> halo;
+  };
+  std::vector<Part> parts(nparts);
+  over_parts([&](int32_t b0, int32_t b1) {
+    std::vector<Rec> cls[3];
+    std::vector<int32_t> halo_at(T, -1);
+    for (int32_t b = b0; b < b1; ++b) {
+      for (auto& c : cls) c.clear();
+      Part& p = parts[b];
+      for (int64_t q = first(b); q < first(b + 1); ++q) {
+        const int64_t c = m.perm[out.cells[q]];
+        for (int k = 0; k < 3; ++k) {
+          const int32_t e = ed.of_half[3 * c + k];
+          const bool right = ed.cL[e] != c;
+          const int64_t o = neighbour(c, k);
+          const bool here = o >= 0 && part[o] == b;
+          if (right && here) continue;
+          const uint32_t self = (uint32_t)k << 14 | (uint32_t)(q - first(b));
+          uint32_t other;
+          int kind = 0;
+          if (o < 0) {
+            other = 0xffffu;
+            kind = 2;
+          } else if (here) {
+            const int64_t co = m.perm[o];
+            int ko = 0;
+            for (int kk = 0; kk < 3; ++kk)
+              if (ed.of_half[3 * co + kk] == e) ko = kk;
+            other = (uint32_t)ko << 14 | (uint32_t)local[o];
+          } else {
+            if (halo_at[o] < 0) {
+              halo_at[o] = (int32_t)p.halo.size();
+              p.halo.push_back((int32_t)o);
+            }
+            other = 3u << 14 | (uint32_t)halo_at[o];
+            kind = 1;
+          }
+          // side A is the edge's left cell
+          cls[kind].push_back({right ? other << 16 | self : self << 16 | other, e});
+        }
+      }
+      for (int32_t o : p.halo) halo_at[o] = -1;
+      for (int kind : {0, 2, 1}) p.recs.insert(p.recs.end(), cls[kind].begin(), cls[kind].end());
+    }
+  });
+  out.halo0.assign(nparts + 1, 0);
+  out.rec0.assign(nparts + 1, 0);
+  for (int32_t b = 0; b < nparts; ++b) {
+    const int32_t nh = (int32_t)parts[b].halo.size(), nr = (int32_t)parts[b].recs.size();
+    out.halo0[b + 1] = out.halo0[b] + nh;
+    out.rec0[b + 1] = out.rec0[b] + nr;
+    out.halo_cap = std::max(out.halo_cap, nh);
+    out.rec_cap = std::max(out.rec_cap, nr);
+  }
+  const size_t H = out.halo0[nparts], R = out.rec0[nparts];
+  out.halo.resize(H);
+  out.halo_pub.resize(H);
+  out.side.resize(R);
+  out.nx.resize(R);
+  out.ny.resize(R);
+  out.len.resize(R);
+  over_parts([&](int32_t b0, int32_t b1) {
+    for (int32_t b = b0; b < b1; ++b) {
+      for (size_t q = 0; q < parts[b].halo.size(); ++q) {
+        const int32_t o = parts[b].halo[q];
+        out.halo[out.halo0[b] + q] = o;
+        out.halo_pub[out.halo0[b] + q] = pub0[part[o]] + local[o];
+      }
+      for (size_t q = 0; q < parts[b].recs.size(); ++q) {
+        const Rec& r = parts[b].recs[q];
+        const size_t at = out.rec0[b] + q;
+        out.side[at] = r.side;
+        out.nx[at] = ed.nx[r.e];
+        out.ny[at] = ed.ny[r.e];
+        out.len[at] = ed.len[r.e];
+      }
+    }
+  });
+  // index 0x3fff of face 3 would read as a wall
+  return out.cell_cap < 0x3fff && out.halo_cap < 0x3fff;
 }
 
 }  // namespace swe

@@ -29,8 +29,31 @@ int guarded(F&& body) noexcept {
 //   < 0, != kWall    local face slot s = -1 - value: face s / tile of tile cell s % tile
 constexpr int32_t kWall = INT32_MIN;
 
+// Edges by caller cell (kept in HostMesh on request): left (lower) and right
+// cell, outward normal and length, and each half-edge's edge.
+struct HostEdges {
+  std::vector<int32_t> cL, cR, of_half;
+  std::vector<double> nx, ny, len;
+};
+
+// Parts of the resident kernel (swe_resident.cuh): part b owns the cells
+// [cell0[b], cell0[b+1]) of `cells` (internal indices, those another part
+// reads first), each with its publication number (or -1); its halo cells
+// (internal index, publication number) and its face records: side codes as
+// two 16-bit halves (side A high), k << 14 | index for face k of the part's
+// cell, k = 3 for a halo cell, 0xffff for a wall.
+struct ResidentParts {
+  std::vector<int32_t> cell0, halo0, rec0;
+  std::vector<int32_t> cells, pub, halo, halo_pub;
+  std::vector<uint32_t> side;
+  std::vector<double> nx, ny, len;
+  int32_t npub = 0;
+  int32_t cell_cap = 0, halo_cap = 0, rec_cap = 0;
+};
+
 struct HostMesh {
   int64_t V = 0, T = 0, E = 0, Eb = 0;
+  HostEdges edges;  // with keep_edges
   // perm[j] = caller index of internal cell j; iperm is its inverse.
   std::vector<int32_t> perm, iperm;
   // Internal-order cell data (FP64).
@@ -82,6 +105,17 @@ constexpr int kRecordSlotPad = 3;
 // at a time spread their shared-memory accesses over the banks (see
 // order_records_for_banks); results do not depend on the order.
 int build_host_mesh(const double* xy, int64_t V, const int32_t* tri, int64_t T, int order,
-                    int32_t tile, bool with_edges, HostMesh& out, bool bank_order = false);
+                    int32_t tile, bool with_edges, HostMesh& out, bool bank_order = false,
+                    bool keep_edges = false);
+
+// The bank order of build_host_mesh's bank_order, applied afterwards to every
+// tile (host threads over tiles).
+void order_records_for_banks(HostMesh& m);
+
+// Cuts a mesh built with keep_edges into nparts parts of nearly equal size,
+// consecutive in the Morton order of the centroids (whatever order the mesh
+// has). Returns false if a part does not fit the record's 14-bit indices.
+bool build_resident_parts(const HostMesh& m, const double* xy, const int32_t* tri, bool is_morton,
+                          int32_t nparts, ResidentParts& out);
 
 }  // namespace swe

@@ -124,11 +124,17 @@ using namespace swe_host;
 namespace {
 
 constexpr int kStepsPerGraph = 16;
+// Most steps of one resident launch, and of one such launch of swe_advance
+// (whose host side reads the clock between launches).
+constexpr int64_t kStepsPerResident = 4096;
 // Default cells per tile: 512 for FP32 (fewer faces computed twice and less
 // per-tile work than 256, one block of 256 threads), 256 for FP64 (whose
 // tiles take twice the shared memory).
 constexpr int kDefaultTileF32 = 512;
 constexpr int kDefaultTileF64 = 256;
+// No mesh above this many cells fits the resident kernel (the chip's shared
+// memory holds about 330,000 FP32 or 175,000 FP64 cells).
+constexpr int64_t kResidentCells = 400000;
 constexpr int64_t kEnsembleWaves = 3;  // waves of work chunks for several scenarios
 
 #define cuda_failed(call) swe_host::cuda_failed_at((call), #call, __FILE__, __LINE__)
@@ -333,13 +339,14 @@ void launch_one_step(swe_state* s, cudaStream_t st) {
   s->walk_back = !s->walk_back;
 }
 
-// CFL step (kind swe::kCflOnly) or mass only (swe::kMassOnly, tiled
-// meshes) of the current state.
+// CFL step (kind swe::kCflOnly) or mass only (swe::kMassOnly) of the current
+// state.
 template <typename Real>
 void launch_cfl(const swe_state* s, int kind = swe::kCflOnly) {
   const swe_mesh* m = s->mesh;
   if (m->kernel == SWE_KERNEL_EDGE)
-    swe::k_cfl<Real><<<m->grid_cfl, 256, 0, m->stream>>>(dev_mesh<Real>(m), dev_state<Real>(s), num_of(m));
+    swe::k_cfl<Real><<<m->grid_cfl, 256, 0, m->stream>>>(dev_mesh<Real>(m), dev_state<Real>(s), num_of(m),
+                                                        kind);
   else
     swe::k_cfl_tiled<Real><<<(int)m->nchunks, 256, 0, m->stream>>>(dev_mesh<Real>(m), dev_state<Real>(s),
                                                                   num_of(m), m->tile, kind);
@@ -419,9 +426,21 @@ swe_status ensure_graph(swe_state* s) {
   return SWE_OK;
 }
 
-// Queues n steps: whole graphs, then single launches for the remainder.
+// Queues n steps: launches of the resident kernel where the mesh has its
+// parts, else whole graphs, then single launches for the remainder.
 swe_status queue_steps(swe_state* s, int64_t n) {
   cudaStream_t st = s->mesh->stream;
+  if (s->mesh->res.nblocks > 0) {
+    while (n > 0) {
+      const int64_t k = std::min(n, kStepsPerResident);
+      if (launch_resident(s, k, st) != cudaSuccess) {
+        cudaGetLastError();  // e.g. its blocks cannot all be resident: one step per launch
+        break;
+      }
+      n -= k;
+    }
+    if (n <= 0) return SWE_OK;
+  }
   if (n >= kStepsPerGraph) {
     swe_status r = ensure_graph(s);
     if (r != SWE_OK) return r;
@@ -576,7 +595,9 @@ swe_status create_batch(int32_t n, const double* const* xy, const int64_t* n_nod
   if (!out) return SWE_EINVAL;
   *out = nullptr;
   if (n <= 0 || !xy || !n_nodes || !tri || !n_tris) return SWE_EINVAL;
+  int64_t all_tris = 0;
   for (int i = 0; i < n; ++i) {
+    all_tris += n_tris[i];
     if (n_tris[i] == 0) return SWE_EMESH;
     if (!xy[i] || !tri[i] || n_nodes[i] <= 0 || n_tris[i] < 0) return SWE_EINVAL;
   }
@@ -592,6 +613,12 @@ swe_status create_batch(int32_t n, const double* const* xy, const int64_t* n_nod
   const int kernel = p.kernel;
   if (kernel == SWE_KERNEL_EDGE && n > 1) return SWE_EINVAL;
   const int tile = p.tile;
+  // The resident kernel runs meshes whose shape the caller left to the
+  // library, if they fit in the chip's shared memory.
+  const bool own_shape = autok && !ghost && (!params || (params->tile == 0 && params->stages == 0 &&
+                                                         params->cells_per_thread == 0 &&
+                                                         params->halo_schedule == 0));
+  const bool keep_edges = own_shape && all_tris <= kResidentCells;
 
   // Host-side construction and validation first (scenarios on parallel host
   // threads): no device is touched for an invalid mesh.
@@ -606,7 +633,8 @@ swe_status create_batch(int32_t n, const double* const* xy, const int64_t* n_nod
         rc[i] = swe::build_host_mesh(xy[i], n_nodes[i], tri[i], n_tris[i], p.order,
                                      kernel == SWE_KERNEL_TILED ? tile : 0,
                                      kernel == SWE_KERNEL_EDGE, hm[i],
-                                     kernel == SWE_KERNEL_TILED && p.precision == SWE_F32);
+                                     kernel == SWE_KERNEL_TILED && p.precision == SWE_F32 && !keep_edges,
+                                     keep_edges);
     };
     std::vector<std::thread> pool;
     try {  // the calling thread takes every scenario no worker takes
@@ -729,6 +757,12 @@ swe_status create_batch(int32_t n, const double* const* xy, const int64_t* n_nod
   }
   m->max_grid = (int)std::max<int64_t>(std::max(m->grid_cell, m->grid_cfl), m->nchunks);
 
+  if (keep_edges && m->T <= (int64_t)sms * resident_max_cells(m)) resident_build(m, hm, xy, tri);
+  // The bank order of the FP32 tiles was left out where the resident kernel
+  // might step the mesh.
+  if (keep_edges && m->res.nblocks == 0 && kernel == SWE_KERNEL_TILED && p.precision == SWE_F32)
+    for (swe::HostMesh& h : hm) swe::order_records_for_banks(h);
+
   // Device layout.
   const int64_t T = m->T, Tp = m->Tp, E = m->E, R = recs, H = halos;
   const int64_t C = m->nchunks;
@@ -758,7 +792,16 @@ swe_status create_batch(int32_t n, const double* const* xy, const int64_t* n_nod
     L.add(sizeof(swe::Chunk) * C);  // and backwards
     if (m->layout.hreg) L.add(4 * tiles * (int64_t)m->layout.halo_cap);
   }
-  if (cudaMalloc((void**)&m->arena.base, L.total) != cudaSuccess) {
+  const size_t bare = L.total;
+  if (m->res.nblocks > 0) L.add(m->res.blob.size());
+  cudaError_t got = cudaMalloc((void**)&m->arena.base, L.total);
+  if (got != cudaSuccess && m->res.nblocks > 0) {  // without the resident kernel's parts
+    cudaGetLastError();
+    m->res = ResidentMesh();
+    L.total = bare;
+    got = cudaMalloc((void**)&m->arena.base, L.total);
+  }
+  if (got != cudaSuccess) {
     cudaGetLastError();
     swe_mesh_destroy(m);
     return SWE_ENOMEM;
@@ -953,6 +996,7 @@ swe_status create_batch(int32_t n, const double* const* xy, const int64_t* n_nod
       chk(upload(m, hpad, m->hpad));
     }
   }
+  if (st == SWE_OK && m->res.nblocks > 0) chk(resident_upload(m));
   if (st != SWE_OK) {
     swe_mesh_destroy(m);
     return st;
@@ -961,12 +1005,13 @@ swe_status create_batch(int32_t n, const double* const* xy, const int64_t* n_nod
   return SWE_OK;
 }
 
-// Integrates every scenario's mass into its control word. The tiled step
-// does not integrate it; k_cfl_tiled does, from the current state, leaving
-// the step control (time step, end-time clamp, stop flag) as it is.
+// Integrates every scenario's mass into its control word. The tiled and the
+// resident step do not integrate it; k_cfl_tiled (k_cfl on separate arrays)
+// does, from the current state, leaving the step control (time step,
+// end-time clamp, stop flag) as it is.
 void refresh_mass(const swe_state* s) {
   const swe_mesh* m = s->mesh;
-  if (m->kernel == SWE_KERNEL_TILED) {
+  if (m->kernel == SWE_KERNEL_TILED || m->res.nblocks > 0) {
     if (m->prm.precision == SWE_F64) launch_cfl<double>(s, swe::kMassOnly);
     else launch_cfl<float>(s, swe::kMassOnly);
   }
@@ -1165,6 +1210,9 @@ swe_status state_init(swe_mesh* m, const double* h, const double* hu, const doub
   L.add(8 * T);                                 // staging
   const bool with_hlo = m->prm.compensated_depth != 0;
   if (with_hlo) L.add(4 * Tp);                  // depth residual (FP32)
+  const size_t xbuf = 2 * (size_t)m->res.npub * (w == 8 ? 32 : 16);  // resident kernel's exchange
+  const size_t slots = 2 * (size_t)m->res.nblocks * 16;
+  if (m->res.nblocks > 0) { L.add(xbuf); L.add(slots); L.add(4 * (size_t)n); }
   L.add(sizeof(swe::Ctl) * n);
   if (cudaMalloc((void**)&s->arena.base, L.total) != cudaSuccess) {
     cudaGetLastError();
@@ -1198,6 +1246,11 @@ swe_status state_init(swe_mesh* m, const double* h, const double* hu, const doub
   s->partial = (double*)s->arena.take(8 * (size_t)m->max_grid);
   s->stage = (double*)s->arena.take(8 * T);
   if (with_hlo) s->hlo = s->arena.take(4 * Tp);
+  if (m->res.nblocks > 0) {
+    s->res_xbuf = (unsigned char*)s->arena.take(xbuf);
+    s->res_slots = (unsigned char*)s->arena.take(slots);
+    s->res_epoch = (uint32_t*)s->arena.take(4 * (size_t)n);
+  }
   s->ctl = (swe::Ctl*)s->arena.take(sizeof(swe::Ctl) * n);
   swe_status st = SWE_OK;
   if (s->arena.overflow) {
@@ -1294,10 +1347,9 @@ swe_status swe_step(swe_state* s, double* dt_used) {
   if (!s) return SWE_EINVAL;
   swe_status st = swe_sync(s);
   if (st != SWE_OK) return st;
-  cudaStream_t str = s->mesh->stream;
   open_end(s);
-  launch_one_step(s, str);
-  CK(cudaGetLastError());
+  st = queue_steps(s, 1);
+  if (st != SWE_OK) return st;
   st = read_ctl(s);
   if (st != SWE_OK) return st;
   if (dt_used) *dt_used = s->host_ctl[0].dt_last;
@@ -1307,7 +1359,8 @@ swe_status swe_step(swe_state* s, double* dt_used) {
 swe_status swe_run(swe_state* s, int64_t n_steps) {
   if (!s || n_steps < 0) return SWE_EINVAL;
   open_end(s);
-  if (n_steps == 0) return ensure_graph(s);  // prepare the graph, take no step
+  if (n_steps == 0)  // prepare the graph (resident meshes use none), take no step
+    return s->mesh->res.nblocks > 0 ? SWE_OK : ensure_graph(s);
   return queue_steps(s, n_steps);
 }
 
@@ -1319,13 +1372,12 @@ swe_status swe_advance(swe_state* s, double t_end, int64_t* n_steps) {
   set_end(s, t_end);
   s->open_ended = false;
   CK(cudaGetLastError());
-  for (;;) {
+  do {  // launches that find the end time reached take no step
+    st = queue_steps(s, s->mesh->res.nblocks > 0 ? kStepsPerResident : kStepsPerGraph);
+    if (st != SWE_OK) return st;
     st = read_ctl(s);
     if (st != SWE_OK) return st;
-    if (all_done(s)) break;
-    st = queue_steps(s, kStepsPerGraph);
-    if (st != SWE_OK) return st;
-  }
+  } while (!all_done(s));
   if (n_steps) *n_steps = s->host_ctl[0].steps - start;
   return status_all(s);
 }

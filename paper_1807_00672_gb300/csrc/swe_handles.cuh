@@ -8,6 +8,11 @@
 
 #include "../../include/swe.h"
 #include "swe_kernels.cuh"
+#include "swe_resident.cuh"
+
+namespace swe {
+struct HostMesh;
+}
 
 namespace swe_host {
 
@@ -51,6 +56,19 @@ struct Scenario {
   int64_t chunk0 = 0, nchunks = 0;  // work chunks (= mass partial slots) of the tiled kernel
 };
 
+// Parts and launch shape of the resident kernel (nblocks 0: the mesh does not
+// take it). The plan arrays lie in one piece of the mesh's arena at `base`;
+// `blob` holds them until they are uploaded.
+struct ResidentMesh {
+  int32_t nblocks = 0, npub = 0;
+  int threads = 0;
+  swe::ResLayout layout{};
+  char* base = nullptr;
+  size_t at_blocks = 0, at_cells = 0, at_pub = 0, at_halo = 0, at_halo_pub = 0, at_rec = 0,
+         at_geo[3] = {0, 0, 0};
+  std::vector<char> blob;
+};
+
 }  // namespace swe_host
 
 struct swe_mesh {
@@ -88,6 +106,7 @@ struct swe_mesh {
   swe::Chunk* chunks_pool = nullptr;  // k_tiled_step's chunks with tile pools
   swe::Chunk* chunks_pool_back = nullptr;  // the same, walked backwards
   bool pooled = false;  // the step launches the pooled k_tiled_step on chunks_pool*
+  swe_host::ResidentMesh res;
   int grid_edge = 1, grid_cell = 1, grid_cfl = 1, max_grid = 1;
   // Handles that use this mesh (states). swe_mesh_destroy while some are
   // alive only marks the mesh; the last of them to go frees it.
@@ -107,6 +126,9 @@ struct swe_state {
   double* stage = nullptr;       // T doubles in caller order
   swe::Ctl* ctl = nullptr;       // one per scenario
   swe::Ctl* host_ctl = nullptr;  // pinned mirror
+  // exchange of the resident kernel's blocks (meshes with res.nblocks > 0)
+  unsigned char *res_xbuf = nullptr, *res_slots = nullptr;
+  uint32_t* res_epoch = nullptr;
   cudaStream_t capture = nullptr;
   cudaGraphExec_t graph = nullptr;
   bool open_ended = true;  // the device t_end is +inf for every scenario
@@ -179,6 +201,15 @@ void launch_forward(const swe_mesh* m, const swe::DevState<float>& ds, cudaStrea
                     bool back = false);
 void launch_forward(const swe_mesh* m, const swe::DevState<double>& ds, cudaStream_t st,
                     bool back = false);
+// Resident kernel (swe_resident.cu). The most cells one block can keep;
+// resident_build cuts a mesh whose host meshes kept their edges into parts
+// (m->res.nblocks stays 0 if they do not fit), resident_upload copies them
+// into the mesh's arena; one launch of up to n steps.
+int64_t resident_max_cells(const swe_mesh* m);
+void resident_build(swe_mesh* m, const std::vector<swe::HostMesh>& hm, const double* const* xy,
+                    const int32_t* const* tri);
+swe_status resident_upload(swe_mesh* m);
+cudaError_t launch_resident(const swe_state* s, int64_t n, cudaStream_t st);
 // Caller order (FP64) -> internal order in the mesh precision, and back;
 // stride 4 for interleaved cells.
 void gather_any(const swe_mesh* m, const double* src, void* dst, int stride);

@@ -1,0 +1,160 @@
+"""Meshes whose tile shape is left to the library and that fit in the chip's
+shared memory take the resident kernel (many steps per launch). Its results
+are those of the one-step tiled kernel (the same arithmetic per face and
+cell, and the same dt sequence): equal bit for bit, over sizes from one cell
+to the largest that fits, both precisions, every cell order, ensembles, the
+depth residual, any split of a run into calls, and end times."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1807_00672_gb300 import inputs, swe
+
+from gpu_util import ensure_built, field_errors, oracle_run
+
+pytestmark = pytest.mark.gpu
+
+
+def pair(case, prec, order="morton", residual=False, tile=256):
+    ensure_built()
+    out = []
+    for kw in (dict(), dict(kernel="tiled", tile=tile)):
+        mesh = swe.Mesh(case.mesh.xy, case.mesh.tri, precision=prec, order=order,
+                        compensated_depth=residual, **kw)
+        out.append(swe.State(mesh, case.h, case.hu, case.hv, case.z, case.n))
+    return out
+
+
+def assert_same(a, b, what=""):
+    for name, x, y in zip(("h", "hu", "hv"), a.fields(), b.fields()):
+        assert np.array_equal(x, y), (what, name, np.abs(x - y).max())
+    assert a.info() == b.info(), what
+    assert a.next_dt() == b.next_dt() and a.t == b.t, what
+
+
+def small_case(nx, ny, seed):
+    return inputs.random_flow_case(nx=nx, ny=ny, lx=10.0 * nx, ly=10.0 * ny, seed=seed,
+                                   jitter=0.3 if min(nx, ny) > 1 else 0.0)
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("nx,ny", [(1, 1), (1, 7), (9, 5), (33, 23), (151, 8), (97, 101)])
+def test_same_bits_as_the_tiled_step(prec, nx, ny):
+    a, b = pair(small_case(nx, ny, 3 + nx), prec)
+    for n in (1, 2, 17, 40):
+        a.run(n)
+        b.run(n)
+        assert_same(a, b, (nx, ny, n))
+    assert a.step() == b.step()
+    assert_same(a, b)
+
+
+@pytest.mark.parametrize("prec,nx,ny", [("f64", 410, 205), ("f32", 560, 280), ("f64", 420, 211),
+                                        ("f32", 570, 291), ("f64", 300, 131)])
+def test_same_bits_at_the_largest_sizes(prec, nx, ny):
+    a, b = pair(small_case(nx, ny, 5), prec)
+    a.run(12)
+    b.run(12)
+    assert_same(a, b)
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("order", ["none", "rcm"])
+def test_other_cell_orders(prec, order):
+    case = inputs.humps_case(nx=61, ny=33, lx=2_000.0, ly=1_000.0, seed=45)
+    a, b = pair(case, prec, order)
+    a.run(60)
+    b.run(60)
+    assert_same(a, b, order)
+    assert a.mass == pytest.approx(b.mass, rel=1e-13 if prec == "f64" else 1e-7)
+
+
+def test_depth_residual():
+    a, b = pair(inputs.water_drop_case(n=71), "f32", residual=True, tile=512)
+    for n in (1, 50):
+        a.run(n)
+        b.run(n)
+        assert_same(a, b)
+    assert a.mass == pytest.approx(b.mass, rel=1e-12)
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+def test_end_times(prec):
+    """advance to an end time, in pieces and past it, and a run after it."""
+    a, b = pair(inputs.three_mounds_case(nx=60, ny=24), prec)
+    assert a.advance(0.31) == b.advance(0.31) > 1
+    assert a.t == 0.31
+    assert_same(a, b)
+    assert a.advance(0.31) == 0
+    assert a.advance(0.8) == b.advance(0.8)
+    a.run(3)
+    b.run(3)
+    assert_same(a, b)
+    case = inputs.stoker_case()
+    ref = oracle.state_from_case(case)
+    k = ref.advance(2.0)
+    st = pair(case, "f64")[0]
+    assert st.advance(2.0) == k and st.t == 2.0
+    assert max(field_errors(st, ref)[0].values()) <= 1e-11
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+def test_ensembles_and_scenarios_that_stop_apart(prec):
+    ensure_built()
+    cases = [inputs.stoker_case(nx=10 + 13 * i, ny=3 + 2 * i, lx=20.0 + 9 * i, seed=i) for i in range(5)]
+    cat = lambda f: np.concatenate([getattr(c, f) for c in cases])
+    sts = []
+    for kw in (dict(), dict(kernel="tiled", tile=128)):
+        mesh = swe.Mesh.ensemble([(c.mesh.xy, c.mesh.tri) for c in cases], precision=prec, **kw)
+        sts.append(swe.State(mesh, cat("h"), cat("hu"), cat("hv"), cat("z"), cat("n")))
+    for st in sts:
+        st.run(20)
+    assert_same(*sts)
+    for st in sts:
+        st.advance(2.0)
+    assert_same(*sts)
+    for i in range(5):
+        x, y = sts[0].scenario(i), sts[1].scenario(i)
+        assert x.pop("mass") == pytest.approx(y.pop("mass"), rel=1e-13 if prec == "f64" else 1e-7)
+        assert x == y and x["t"] == 2.0
+
+
+def test_reset_states_and_two_states_on_one_mesh():
+    """A state set anew after runs of any length starts clean (the exchange
+    words of earlier launches are never taken for new ones)."""
+    case = inputs.humps_case(nx=61, ny=33, lx=2_000.0, ly=1_000.0, seed=45)
+    a, b = pair(case, "f32")
+    c = swe.State(a.mesh, case.h, case.hu, case.hv, case.z, case.n)
+    b.run(10)
+    for n in (1, 2, 3, 10):
+        a.run(n)
+        c.run(3)
+        a.set(case.h, case.hu, case.hv)
+        a.run(10)
+        assert_same(a, b, n)
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+def test_errors_are_latched(prec):
+    case = inputs.random_flow_case(nx=37, ny=23, seed=41)
+    ensure_built()
+    mesh = swe.Mesh(case.mesh.xy, case.mesh.tri, precision=prec, wait_rounds=-1)
+    st = swe.State(mesh, case.h, case.hu, case.hv, case.z, case.n)
+    for _ in range(2):
+        with pytest.raises(swe.SweError) as ei:
+            st.run(5)
+        assert ei.value.status == swe.SWE_ETIMEOUT
+    assert st.info()["steps"] == 0
+    # momentum whose square overflows: SWE_ENAN from both kernels
+    case.hu[100] = 1e30 if prec == "f32" else 1e200
+    case.n[:] = 0.0
+    for st in pair(case, prec):
+        with pytest.raises(swe.SweError) as ei:
+            st.run(30)
+        assert ei.value.status == swe.SWE_ENAN
+    # a state set anew clears it
+    ref, _ = oracle_run(inputs.random_flow_case(nx=37, ny=23, seed=41), 20)
+    ok = inputs.random_flow_case(nx=37, ny=23, seed=41)
+    st = pair(ok, "f64")[0]
+    st.run(20)
+    assert max(field_errors(st, ref)[0].values()) <= 1e-11
