@@ -127,15 +127,27 @@ constexpr int kStepsPerGraph = 16;
 // Most steps of one resident launch, and of one such launch of swe_advance
 // (whose host side reads the clock between launches).
 constexpr int64_t kStepsPerResident = 4096;
-// Default cells per tile: 512 for FP32 (fewer faces computed twice and less
-// per-tile work than 256, one block of 256 threads), 256 for FP64 (whose
-// tiles take twice the shared memory).
+// Default cells per tile: 256 for FP64 (whose tiles take twice the shared
+// memory). FP32: 512 (fewer faces computed twice and less per-tile work than
+// 256) where every block walks many tiles; 256 for meshes and ensembles up to
+// kSmallTileCells, whose blocks walk few: finer shares even out the SMs.
+// Measured, us per step at 256 and 512: 1.0M cells 19.7 and 20.9, 2.0M 31.5
+// and 33.2, 4.0M 56.2 and 57.4, 10.0M 130.2 and 128.8; 32 scenarios of 2.3M
+// cells 36.7 and 45.3.
 constexpr int kDefaultTileF32 = 512;
+constexpr int kSmallTileF32 = 256;
+constexpr int64_t kSmallTileCells = 6000000;
 constexpr int kDefaultTileF64 = 256;
 // No mesh above this many cells fits the resident kernel (the chip's shared
 // memory holds about 330,000 FP32 or 175,000 FP64 cells).
 constexpr int64_t kResidentCells = 400000;
-constexpr int64_t kEnsembleWaves = 3;  // waves of work chunks for several scenarios
+// Several scenarios: up to kEnsembleWaves waves of work chunks, of at least
+// kWaveTiles tiles each. More waves balance uneven scenarios better, but each
+// block pays its first copies again: 32 scenarios of 2.3M cells (9.7 tiles of
+// 256 cells per resident block) take 36.5 us per step in 1 wave, 40.2 in 2 and
+// 44.6 in 3; 256 scenarios of 26.6M cells (114 tiles) are fastest in 3.
+constexpr int64_t kEnsembleWaves = 3;
+constexpr int64_t kWaveTiles = 12;
 
 #define cuda_failed(call) swe_host::cuda_failed_at((call), #call, __FILE__, __LINE__)
 
@@ -612,13 +624,14 @@ swe_status create_batch(int32_t n, const double* const* xy, const int64_t* n_nod
   if (autok && n == 1 && p.order == SWE_ORDER_RCM && !p.compensated_depth) p.kernel = SWE_KERNEL_EDGE;
   const int kernel = p.kernel;
   if (kernel == SWE_KERNEL_EDGE && n > 1) return SWE_EINVAL;
+  // no shape asked for: the library's own
+  const bool default_shape = !params || (params->tile == 0 && params->stages == 0 &&
+                                         params->cells_per_thread == 0 && params->halo_schedule == 0);
+  if (default_shape && p.precision == SWE_F32 && all_tris <= kSmallTileCells) p.tile = kSmallTileF32;
   const int tile = p.tile;
   // The resident kernel runs meshes whose shape the caller left to the
   // library, if they fit in the chip's shared memory.
-  const bool own_shape = autok && !ghost && (!params || (params->tile == 0 && params->stages == 0 &&
-                                                         params->cells_per_thread == 0 &&
-                                                         params->halo_schedule == 0));
-  const bool keep_edges = own_shape && all_tris <= kResidentCells;
+  const bool keep_edges = default_shape && autok && !ghost && all_tris <= kResidentCells;
 
   // Host-side construction and validation first (scenarios on parallel host
   // threads): no device is touched for an invalid mesh.
@@ -704,11 +717,13 @@ swe_status create_batch(int32_t n, const double* const* xy, const int64_t* n_nod
   const int geo_arrays = (p.precision == SWE_F64) ? 3 : 2;
 
   // Work chunks of the tiled kernels (see swe::Chunk). One scenario: one
-  // wave of resident blocks with ceil(ntiles / resident) tiles each. Several
-  // scenarios: about kEnsembleWaves waves; scenario s is split into
-  // ceil(ntiles_s / per) interleaved chunks, and the chunks are launched
-  // largest first so that the block scheduler, which starts blocks in index
-  // order as slots free up, balances the SMs (longest-processing-time order).
+  // wave of resident blocks, one chunk for every block slot (1.0M cells: 20.9
+  // against 21.9 us per step with chunks of equal tile counts, which leave
+  // slots empty). Several scenarios: up to kEnsembleWaves waves; scenario s is
+  // split into ceil(ntiles_s / per) interleaved chunks, and the chunks are
+  // launched largest first so that the block scheduler, which starts blocks in
+  // index order as slots free up, balances the SMs
+  // (longest-processing-time order).
   std::vector<swe::Chunk> chunks;
   if (kernel == SWE_KERNEL_TILED) {
     const bool want_pipe = p.halo_schedule == 2 && p.precision == SWE_F32 && m->stages == 2;
@@ -730,12 +745,13 @@ swe_status create_batch(int32_t n, const double* const* xy, const int64_t* n_nod
       return SWE_ECUDA;
     }
     const int64_t resident = (int64_t)sms * occ;
-    const int64_t waves = (n == 1) ? 1 : kEnsembleWaves;
+    const int64_t waves =
+        n == 1 ? 1 : std::min(kEnsembleWaves, std::max<int64_t>(1, tiles / (resident * kWaveTiles)));
     const int64_t per = std::max<int64_t>(1, (tiles + resident * waves - 1) / (resident * waves));
     for (int i = 0; i < n; ++i) {
       Scenario& sc = m->scen[i];
       sc.chunk0 = (int64_t)chunks.size();
-      sc.nchunks = (sc.ntiles + per - 1) / per;
+      sc.nchunks = n == 1 ? std::min(tiles, resident) : (sc.ntiles + per - 1) / per;
       for (int64_t r = 0; r < sc.nchunks; ++r) {
         swe::Chunk c{};
         c.scen = i;
