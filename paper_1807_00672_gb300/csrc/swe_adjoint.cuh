@@ -5,13 +5,18 @@
 // semi-implicit friction):
 //   U*_i     = U^n_i - (dt / Omega_i) R_i,  R_i = sum over faces of s l (F + P n)
 //   U^{n+1}_i = friction(U*_i)              (clip of h at 0, momentum / d)
-// Given lambda = dL/dU^{n+1}, the adjoint step forms, per cell,
+// Given lambda = dL/dU^{n+1},
 //   mu_i  = dL/dU*_i          (friction transposed; needs only U^{n+1}, g n^2, dt)
 //   rho_i = dL/dR_i = -(dt / Omega_i) mu_i
 // and per face the vector-Jacobian product of its two residual contributions
-// with (rho_A, rho_B), giving dL/d(h, hu, hv, z) of both sides. Then
-//   dL/dU^n_i = mu_i + sum over the cell's faces of its side's part,
+// with (rho_A, rho_B), giving dL/d(h, u, v, z) of both sides; then
+//   dL/dU^n_i = mu_i + sum over the cell's faces of its side's part
+//               (velocities taken back to hu, hv once per cell),
 //   dL/dz_i  += sum of the z parts,  dL/d(g n^2)_i += friction part.
+// What a step hands to the one before it is mu, not lambda: the cell's own
+// thread has its U^n staged anyway and transposes the friction of step n - 1
+// right there, so no step reads U^{n+1} and a halo cell costs its U^n, mu and
+// area only.
 // Every branch (wet/dry tests, the HLLC case, the min/max of the wave-speed
 // estimates and of the reconstruction) is taken as the forward step takes
 // it; where the forward picks between two equal values (a tie of max(zA, zB)
@@ -29,210 +34,262 @@
 
 namespace swe {
 
+// dt h^{-7/3} and 1 / h of a wet depth.
+__device__ __forceinline__ void depth_powers(float h, float dt, float& ch, float& rh) {
+  ch = Ops<float>::friction(dt, 1.0f, 1.0f, h);
+  rh = rcp_approx(h);
+}
+__device__ __forceinline__ void depth_powers(double h, double dt, double& ch, double& rh) {
+  const double y = icbrt_nr(h), y2 = mul_rn(y, y);
+  rh = mul_rn(y2, y);
+  ch = mul_rn(dt, mul_rn(mul_rn(y2, y2), rh));
+}
+
+// Signs by value; FP64 from the bit patterns (a comparison costs as much of
+// the FP64 pipe as a multiply-add).
+__device__ __forceinline__ bool below0(float x) { return x < 0.0f; }
+__device__ __forceinline__ bool below0(double x) {
+  return (unsigned long long)__double_as_longlong(x) > 0x8000000000000000ull;
+}
+__device__ __forceinline__ bool above0(float x) { return x > 0.0f; }
+__device__ __forceinline__ bool above0(double x) { return __double_as_longlong(x) > 0; }
+// a >= b
+__device__ __forceinline__ bool at_least(float a, float b) { return a >= b; }
+__device__ __forceinline__ bool at_least(double a, double b) {
+  const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b);
+  const long long ka = ia ^ ((ia >> 63) & 0x7fffffffffffffffll);
+  const long long kb = ib ^ ((ib >> 63) & 0x7fffffffffffffffll);
+  return ka >= kb || ((ia | ib) << 1) == 0;  // -0 and +0 are equal
+}
+// 2 x for a normal x > 0 (or 0 with pos false)
+__device__ __forceinline__ float twice(float x, bool) { return x + x; }
+__device__ __forceinline__ double twice(double x, bool pos) {
+  return pos ? __hiloint2double(__double2hiint(x) + 0x00100000, __double2loint(x)) : 0.0;
+}
+
 // dL/dU* of one cell from its post-step state (h1, q1x, q1y) and lambda:
-// mu (3 values) and the derivative with respect to its g n^2.
+// mu (3 values) and the derivative with respect to its g n^2 (left 0 where
+// g n^2 is 0: it only enters dL/dn, multiplied by n).
 template <typename Real>
 __device__ __forceinline__ void cell_vjp(Real h1, Real q1x, Real q1y, Real lh, Real lx, Real ly,
                                          Real gn2, Real dt, const Num& num, Real& mh, Real& mx,
                                          Real& my, Real& bgn2) {
   using O = Ops<Real>;
   const Real zero = Real(0);
-  if (O::wet(h1, num)) {
-    const Real q1n = O::sqrt_(q1x * q1x + q1y * q1y);
-    const Real ch = O::friction(dt, Real(1), Real(1), h1);  // dt h^{-7/3}
-    const Real c = ch * gn2;
-    const Real cq = c * q1n;        // (d - 1) / d
-    const Real rd = Real(1) - cq;   // 1 / d
-    const Real ql = q1x * lx + q1y * ly;
-    const Real k = q1n > zero ? O::div(c * ql, q1n) : zero;
-    mx = rd * (lx - k * q1x);
-    my = rd * (ly - k * q1y);
-    mh = lh + Real(7.0 / 3.0) * O::div(cq, h1) * ql;
-    bgn2 = -q1n * ch * ql;
-  } else {
-    mh = lh;
-    mx = zero;
-    my = zero;
-    bgn2 = zero;
-  }
+  mh = lh;
+  mx = zero;
+  my = zero;
+  bgn2 = zero;
+  if (!O::wet(h1, num)) return;
+  mx = lx;
+  my = ly;
+  if (!above0(gn2)) return;
+  const Real q1n = O::sqrt_(fma_rn(q1x, q1x, q1y * q1y));
+  Real ch, rh;
+  depth_powers(h1, dt, ch, rh);
+  const Real c = ch * gn2;
+  const Real cq = c * q1n;        // (d - 1) / d
+  const Real rd = Real(1) - cq;   // 1 / d
+  const Real ql = fma_rn(q1x, lx, q1y * ly);
+  const Real k = above0(q1n) ? O::div(c * ql, q1n) : zero;
+  mx = rd * fma_rn(-k, q1x, lx);
+  my = rd * fma_rn(-k, q1y, ly);
+  mh = fma_rn(Real(7.0 / 3.0) * (cq * rh), ql, lh);
+  bgn2 = -(q1n * ch) * ql;
 }
 
 // Vector-Jacobian product of one face, with both sides' contributions:
-// inputs the sides' cells (h, hu, hv, z) as the forward step read them, the
-// geometry, and rho = dL/dR of side A (the face adds c_A to R_A) and side B
-// (the face subtracts c_B from R_B); outputs gA, gB = dL/d(h, hu, hv, z) of
-// each side through this face. The face is the clamped form of the flux the
-// tiled steps compute (face_flux_f32, face_flux_f64): one HLL formula with
-// the clamped speeds S- = min(S_A, 0), S+ = max(S_B, 0), the dry side's
-// normal velocity replaced by un_B - 2 c_B (or un_A + 2 c_A) in the
-// wave-speed estimates, the transverse momentum upwinded by the sign of F0.
-// It is the same function of the inputs as the HLLC case analysis (the
-// clamped speeds reproduce the supersonic cases: with S_A >= 0, S- = 0 and
-// F = F_A, whose derivative with respect to S_A is 0), so the derivatives
-// agree with the case analysis's away from ties; it has no case branches.
-// Ties follow fixed conventions: max(zA, zB) and the speed estimates take
-// the first argument, S_A = 0 counts as S_A >= 0 and S_B = 0 as S_B <= 0.
-// For a wall B is ignored (the mirror of A folds into gA, gB = 0).
+// inputs the sides' cells (h, u, v, z) as the forward step reads them
+// (velocities formed once per cell, 0 on a dry one), the geometry, and rho =
+// dL/dR of side A (the face adds c_A to R_A) and side B (the face subtracts
+// c_B from R_B); outputs gA, gB = dL/d(h, u, v, z) of each side through this
+// face. The face is the clamped form of the flux the tiled steps compute
+// (face_flux_f32, face_flux_f64): one HLL formula with the clamped speeds
+// S- = min(S_A, 0), S+ = max(S_B, 0), the dry side's normal velocity replaced
+// by un_B - 2 c_B (or un_A + 2 c_A) in the wave-speed estimates, the
+// transverse momentum upwinded by the sign of F0. It is the same function of
+// the inputs as the HLLC case analysis (the clamped speeds reproduce the
+// supersonic cases: with S_A >= 0, S- = 0 and F = F_A, whose derivative with
+// respect to S_A is 0), so the derivatives agree with the case analysis's
+// away from ties; it has no case branches. Ties follow fixed conventions:
+// max(zA, zB) and the speed estimates take the first argument, S_A = 0 counts
+// as S_A >= 0 and S_B = 0 as S_B <= 0. For a wall B is ignored (the mirror of
+// A folds into gA, gB = 0).
+//
+// FP64: the FP64 pipe bounds the adjoint as it bounds the step, so the sweep
+// is arranged for few FP64 instructions (115 of them; about 175 when each
+// face formed its velocities and differentiated N / D):
+//   - with D = S+ - S-, and w- = S- / D, w+ = S+ / D, w = S- S+ / D, F_k of
+//     side values f and states q is w+ f_A - w- f_B + w (q_B - q_A), and its
+//     derivatives are dF/dS+ = w- (df - S- dq) / D and dF/dS- = -w+ (df - S+ dq) / D
+//     (df, dq: B minus A), so neither numerator is formed;
+//   - the wave speeds as in face_flux_f64, from their distance to un -+ c;
+//   - z enters through the higher side only: one side's part, negated for
+//     the other;
+//   - signs and orders from bit patterns.
 template <typename Real, bool Wall>
-__device__ __forceinline__ void face_vjp_clamped(const V4<Real>& A, const V4<Real>& B, Real nx,
-                                                 Real ny, Real len, const Num& num, Real rA0,
-                                                 Real rA1, Real rA2, Real rB0, Real rB1, Real rB2,
-                                                 Real gA[4], Real gB[4]) {
+__device__ __forceinline__ void face_vjp(const V4<Real>& A, const V4<Real>& B, Real nx, Real ny,
+                                         Real len, const Num& num, Real rA0, Real rA1, Real rA2,
+                                         Real rB0, Real rB1, Real rB2, Real gA[4], Real gB[4]) {
   using O = Ops<Real>;
-  const Real zero = Real(0), half = Real(0.5), quarter = Real(0.25);
-  const Real g = Real(num.g), hg = half * g;
-  // ---- forward, keeping what the reverse sweep needs
-  const Real rA = O::wet(A.x, num) ? O::div(Real(1), A.x) : zero;  // 0 on a dry cell
-  const Real uA = A.y * rA, vA = A.z * rA;
-  const Real unA = uA * nx + vA * ny;
-  const Real utA = vA * nx - uA * ny;
-  Real hB, zB, unB, utB, uB = zero, vB = zero, rB = zero;
-  if (Wall) {
-    hB = A.x; zB = A.w; unB = -unA; utB = utA;
-  } else {
-    rB = O::wet(B.x, num) ? O::div(Real(1), B.x) : zero;
-    uB = B.y * rB;
-    vB = B.z * rB;
-    hB = B.x; zB = B.w;
-    unB = uB * nx + vB * ny;
-    utB = vB * nx - uB * ny;
-  }
-  const bool zsA = A.w >= zB;  // max(zA, zB) taken from A on a tie
+  const Real zero = Real(0), k34 = Real(0.75), two = Real(2);
+  const Real g = Real(num.g), hg = Real(0.5) * g;
+  // ---- forward
+  const Real unA = fma_rn(A.y, nx, A.z * ny);
+  const Real hB = Wall ? A.x : B.x, zB = Wall ? A.w : B.w;
+  const Real unB = Wall ? -unA : fma_rn(B.y, nx, B.z * ny);
+  const bool zsA = Wall || at_least(A.w, zB);  // max(zA, zB) taken from A on a tie
   const Real zs = zsA ? A.w : zB;
-  const Real xA = A.x + A.w - zs, xB = hB + zB - zs;
+  const Real xA = sub_rn(add_rn(A.x, A.w), zs), xB = Wall ? xA : sub_rn(add_rn(hB, zB), zs);
   const bool wetA = O::wet(xA, num), wetB = O::wet(xB, num);  // reconstructed sides wet
   const Real hAs = wetA ? xA : zero, hBs = wetB ? xB : zero;
-  const Real cA = O::sqrt_(g * hAs), cB = O::sqrt_(g * hBs);
-  const Real vnA = wetA ? unA : unB - Real(2) * cB;
-  const Real vnB = wetB ? unB : unA + Real(2) * cA;
-  const Real us = (vnA + vnB) * half + cA - cB;
-  const Real cs = (cA + cB) * half + (vnA - vnB) * quarter;
-  const Real a1 = vnA - cA, a2 = us - cs, b1 = vnB + cB, b2 = us + cs;
-  const bool firstA = a1 <= a2, firstB = b1 >= b2;
-  const Real SA = firstA ? a1 : a2, SB = firstB ? b1 : b2;
-  const bool negA = SA < zero, posB = SB > zero;
+  const Real pA = hg * hAs, pB = Wall ? pA : hg * hBs;
+  const Real cA = O::sqrt_(twice(pA, wetA)), cB = Wall ? cA : O::sqrt_(twice(pB, wetB));
+  Real vnA = unA, vnB = unB;
+  if (!(wetA && wetB)) {
+    if (!wetA) vnA = fma_rn(-two, cB, unB);
+    if (!wetB) vnB = fma_rn(two, cA, unA);
+  }
+  const Real dv = vnB - vnA, dc = cA - cB;
+  const Real eA = fma_rn(two, dc, dv), eB = fma_rn(two, dc, -dv);
+  const bool secA = below0(eA), secB = above0(eB);  // the star-region estimate is the extreme one
+  const Real SA = fma_rn(k34, secA ? eA : zero, vnA - cA);
+  const Real SB = fma_rn(k34, secB ? eB : zero, vnB + cB);
+  const bool negA = below0(SA), posB = above0(SB);
   const Real Sm = negA ? SA : zero, Sp = posB ? SB : zero;
   const Real qA = hAs * unA, qB = hBs * unB;
-  const Real FA1 = qA * unA + hg * hAs * hAs, FB1 = qB * unB + hg * hBs * hBs;
+  const Real dh = hBs - hAs, dq = qB - qA;
+  const Real dF = Wall ? zero : fma_rn(qB, unB, pB * hBs) - fma_rn(qA, unA, pA * hAs);
   const bool live = wetA || wetB;  // both sides dry: F = 0 whatever the speeds
-  const Real inv = live ? O::div(Real(1), Sp - Sm) : zero;
-  const Real SS = Sm * Sp, dh = hBs - hAs, dq = qB - qA;
-  const Real N0 = Sp * qA - Sm * qB + SS * dh;
-  const Real N1 = Sp * FA1 - Sm * FB1 + SS * dq;
-  const Real F0 = N0 * inv;
-  const bool upA = F0 >= zero;  // transverse momentum from A where F0 >= 0
+  const Real inv = live ? O::rcp(Sp - Sm) : zero;
+  const Real wm = Sm * inv, wp = Sp * inv, ws = Sm * wp;
 
   // ---- reverse sweep
   // residual contributions: A gets +l (F0, Fx + PA nx, Fy + PA ny), B gets
   // -l (F0, Fx + PB nx, Fy + PB ny), Fx = F1 nx - F2 ny, Fy = F1 ny + F2 nx
-  const Real bFx = len * (rA1 - rB1), bFy = len * (rA2 - rB2);
-  const Real bF1 = bFx * nx + bFy * ny;
-  Real bF0 = zero, bF2 = zero;
-  if (!Wall) {
-    bF0 = len * (rA0 - rB0);
-    bF2 = bFy * nx - bFx * ny;
-  }
-  const Real bPA = len * (rA1 * nx + rA2 * ny);
-  const Real bPB = Wall ? zero : -len * (rB1 * nx + rB2 * ny);
+  const Real gx = len * nx, gy = len * ny;
+  const Real d1 = Wall ? rA1 : rA1 - rB1, d2 = Wall ? rA2 : rA2 - rB2;
+  const Real bF1 = fma_rn(d1, gx, d2 * gy);
   // P = g/2 (h^2 - h*^2)
-  Real bhA = g * A.x * bPA, bhB = g * hB * bPB;
-  Real bhAs = -g * hAs * bPA, bhBs = -g * hBs * bPB;
-  // F2 = F0 ut
-  bF0 += bF2 * (upA ? utA : utB);
-  const Real but = bF2 * F0;
-  Real butA = upA ? but : zero, butB = upA ? zero : but;
-  // F0 = N0 / D, F1 = N1 / D, D = S+ - S-
-  const Real bN0 = bF0 * inv, bN1 = bF1 * inv;
-  const Real bD = -(bF0 * N0 + bF1 * N1) * inv * inv;
-  const Real bSp = bD + bN0 * (qA + Sm * dh) + bN1 * (FA1 + Sm * dq);
-  const Real bSm = -bD + bN0 * (Sp * dh - qB) + bN1 * (Sp * dq - FB1);
-  Real bqA = bN0 * Sp - bN1 * SS, bqB = bN1 * SS - bN0 * Sm;
-  bhBs += bN0 * SS;
-  bhAs -= bN0 * SS;
-  const Real bFA1 = bN1 * Sp, bFB1 = -bN1 * Sm;
-  // F1 of each side = q un + g/2 h*^2, q = h* un
-  bqA += bFA1 * unA;
-  bqB += bFB1 * unB;
-  Real bunA = bFA1 * qA + bqA * hAs, bunB = bFB1 * qB + bqB * hBs;
-  bhAs += bFA1 * g * hAs + bqA * unA;
-  bhBs += bFB1 * g * hBs + bqB * unB;
-  // S- = min(S_A, 0), S+ = max(S_B, 0); the speed estimates
-  const Real bSA = negA ? bSm : zero, bSB = posB ? bSp : zero;
-  Real bvnA = zero, bvnB = zero, bcA = zero, bcB = zero, bus = zero, bcs = zero;
-  if (firstA) { bvnA += bSA; bcA -= bSA; } else { bus += bSA; bcs -= bSA; }
-  if (firstB) { bvnB += bSB; bcB += bSB; } else { bus += bSB; bcs += bSB; }
-  bvnA += half * bus + quarter * bcs;
-  bvnB += half * bus - quarter * bcs;
-  bcA += bus + half * bcs;
-  bcB += half * bcs - bus;
-  // a dry side's velocity in the estimates
-  if (wetA) { bunA += bvnA; } else { bunB += bvnA; bcB -= Real(2) * bvnA; }
-  if (wetB) { bunB += bvnB; } else { bunA += bvnB; bcA += Real(2) * bvnB; }
-  // c = sqrt(g h*): dc/dh* = g / (2 c) on a wet side (c = 0 and no term on a dry one)
-  if (wetA) bhAs += bcA * O::div(hg, cA);
-  if (wetB) bhBs += bcB * O::div(hg, cB);
-  // reconstruction h* = h + z - max(zA, zB) where it stays wet
-  Real bzA = zero, bzB = zero, bzs = zero;
-  if (wetA) { bhA += bhAs; bzA += bhAs; bzs -= bhAs; }
-  if (wetB) { bhB += bhBs; bzB += bhBs; bzs -= bhBs; }
-  if (zsA) bzA += bzs; else bzB += bzs;
-  if (Wall) {  // B mirrors A: hB = hA, zB = zA, unB = -unA, utB = utA
-    bhA += bhB;
-    bzA += bzB;
-    bunA -= bunB;
-    butA += butB;
+  const Real gPA = g * (Wall ? bF1 : fma_rn(rA1, gx, rA2 * gy));
+  const Real gPB = Wall ? zero : -g * fma_rn(rB1, gx, rB2 * gy);
+  Real bF0 = zero, but = zero;
+  bool upA = true;
+  if (!Wall) {
+    // F2 = F0 ut, ut of the upwind side
+    const Real F0 = fma_rn(ws, dh, fma_rn(wp, qA, -(wm * qB)));
+    upA = !below0(F0);
+    const Real uu = upA ? A.y : B.y, vv = upA ? A.z : B.z;
+    const Real bF2 = fma_rn(d2, gx, -(d1 * gy));
+    bF0 = fma_rn(bF2, fma_rn(vv, nx, -(uu * ny)), len * (rA0 - rB0));
+    but = bF2 * F0;
   }
-  // face frame -> x, y velocities -> conserved variables (u = hu r, r = 1/h
-  // on a wet cell, 0 on a dry one)
-  const Real buA = bunA * nx - butA * ny, bvA = bunA * ny + butA * nx;
-  gA[0] = bhA - (buA * uA + bvA * vA) * rA;
-  gA[1] = buA * rA;
-  gA[2] = bvA * rA;
-  gA[3] = bzA;
+  // F0 (states q, h) and F1 (states F, q) of the two sides and the speeds
+  const Real P = Wall ? zero : fma_rn(bF1, dF, bF0 * dq) * inv;
+  const Real Q = (Wall ? bF1 * dq : fma_rn(bF1, dq, bF0 * dh)) * inv;
+  const Real bSB = posB ? wm * fma_rn(-Sm, Q, P) : zero;
+  const Real bSA = negA ? wp * fma_rn(Sp, Q, -P) : zero;
+  const Real bFA = bF1 * wp, bFB = -(bF1 * wm), s1 = bF1 * ws, s0 = Wall ? zero : bF0 * ws;
+  const Real bqA = fma_rn(bFA, unA, Wall ? -s1 : fma_rn(bF0, wp, -s1));
+  const Real bqB = fma_rn(bFB, unB, Wall ? s1 : fma_rn(-bF0, wm, s1));
+  Real bunA = fma_rn(bqA, hAs, bFA * qA), bunB = fma_rn(bqB, hBs, bFB * qB);
+  Real bhAs = fma_rn(fma_rn(g, bFA, -gPA), hAs, fma_rn(bqA, unA, -s0));
+  Real bhBs = fma_rn(Wall ? g * bFB : fma_rn(g, bFB, -gPB), hBs, fma_rn(bqB, unB, s0));
+  // the speed estimates
+  const Real tA = secA ? k34 * bSA : zero, tB = secB ? k34 * bSB : zero;
+  const Real td = tA - tB, ts = tA + tB;
+  const Real bvA = bSA - td, bvB = bSB + td;
+  Real bcA = fma_rn(two, ts, -bSA), bcB = fma_rn(-two, ts, bSB);
+  if (wetA && wetB) {
+    bunA += bvA;
+    bunB += bvB;
+  } else {  // a dry side's velocity in the estimates
+    if (wetA) { bunA += bvA; } else { bunB += bvA; bcB = fma_rn(-two, bvA, bcB); }
+    if (wetB) { bunB += bvB; } else { bunA += bvB; bcA = fma_rn(two, bvB, bcA); }
+  }
+  // c = sqrt(g h*): dc/dh* = g / (2 c) on a wet side (c = 0 and no term on a dry one)
+  bhAs = wetA ? fma_rn(bcA * hg, O::rcp(cA), bhAs) : zero;
+  bhBs = wetB ? fma_rn(bcB * hg, Wall ? O::rcp(cA) : O::rcp(cB), bhBs) : zero;
+  // reconstruction h* = h + z - max(zA, zB) where it stays wet
+  Real bhA = fma_rn(A.x, gPA, bhAs);
+  if (Wall) {  // B mirrors A: hB = hA, zB = zA, unB = -unA, utB = utA
+    bhA += bhBs;
+    bunA -= bunB;
+  }
+  // face frame -> x, y
+  const Real tx = but * ny, ty = but * nx;
+  gA[0] = bhA;
+  gA[1] = Wall ? bunA * nx : fma_rn(bunA, nx, upA ? -tx : zero);
+  gA[2] = Wall ? bunA * ny : fma_rn(bunA, ny, upA ? ty : zero);
+  gA[3] = Wall ? zero : (zsA ? -bhBs : bhAs);
   if (Wall) {
     gB[0] = zero; gB[1] = zero; gB[2] = zero; gB[3] = zero;
   } else {
-    const Real buB = bunB * nx - butB * ny, bvB = bunB * ny + butB * nx;
-    gB[0] = bhB - (buB * uB + bvB * vB) * rB;
-    gB[1] = buB * rB;
-    gB[2] = bvB * rB;
-    gB[3] = bzB;
+    gB[0] = fma_rn(hB, gPB, bhBs);
+    gB[1] = fma_rn(bunB, nx, upA ? zero : -tx);
+    gB[2] = fma_rn(bunB, ny, upA ? zero : ty);
+    gB[3] = zsA ? bhBs : -bhAs;
   }
 }
 
-// Inputs and outputs of one adjoint launch (interleaved cells, internal
-// order, padded to whole tiles).
+// Loss seeds of the gauges: the ncells distinct cells that hold gauges, and
+// for each the gauges in it (index[first[c]] .. index[first[c + 1] - 1], in
+// ascending order); seed[k G + j] is dL/d(depth at gauge j after step k).
+struct GaugeSeeds {
+  const int32_t* cells;
+  const int32_t* first;
+  const int32_t* index;
+  const double* seed;
+  int G, ncells;
+};
+
+// Adds the seeds of step k to the depth adjoint of interleaved cells: one
+// thread per distinct cell, so that repeated gauge cells add up in a fixed
+// order. (One thread for all of them: 64 gauges added 16 us to an adjoint
+// step of 1M triangles, 54 us, each a dependent trip to L2.)
+template <typename Real>
+__device__ __forceinline__ void add_gauge_seeds(Real* lam, const GaugeSeeds& g, long long k, int tid,
+                                                int nthreads) {
+  for (int c = tid; c < g.ncells; c += nthreads) {
+    Real* p = lam + 4 * (int64_t)g.cells[c];
+    Real v = __ldcg(p);  // other blocks wrote it
+    for (int q = g.first[c]; q < g.first[c + 1]; ++q) v += Real(g.seed[k * g.G + g.index[q]]);
+    *p = v;
+  }
+}
+
+// Inputs and outputs of one adjoint launch, step n (interleaved cells,
+// internal order, padded to whole tiles).
 template <typename Real>
 struct AdjArgs {
   const Real* un;      // U^n (h, hu, hv, z)
-  const Real* u1;      // U^{n+1} (h, hu, hv, z)
-  const Real* lam_in;  // dL/dU^{n+1} (h, hu, hv, accumulated dL/dz)
-  Real* lam_out;       // dL/dU^n, same layout
+  const Real* mu_in;   // mu of step n (h, hu, hv), accumulated dL/dz
+  Real* mu_out;        // the same of step n - 1; for n = 0 dL/dU^0 and dL/dz
   const Real* gn2;     // g n^2 per cell
   Real* dgn2;          // accumulated dL/d(g n^2) per cell (read-modify-write)
-  Real dt;
+  Real dt, dt_prev;    // time steps of steps n and n - 1
+  int last;            // 1: n = 0
   int* err;            // kErr* bits (timeouts)
-  // Gauge seeds added to the depth adjoint of lam_out once every block is
-  // done (by the last block): lam_out[4 gcells[j]] += gseed[gstep G + j],
-  // j < G; gstep < 0 adds nothing. ticket: a zeroed counter.
-  const int32_t* gcells;
-  const double* gseed;
-  int G;
+  // Gauge seeds of U^n, added to the depth part of mu_out once every block is
+  // done (by the last block); gstep < 0 adds nothing. (The transposed
+  // friction adds its part to the depth derivative, so the seed may come
+  // after it.) ticket: a zeroed counter.
+  GaugeSeeds gauges;
   long long gstep;
   unsigned int* ticket;
 };
 
 // Shared-memory plan of k_tiled_adjoint. Per stage: the tile's and its
-// halo's cells of U^n; the halo cells' U^{n+1}, lambda, areas and g n^2 (a
-// tile's own cells read theirs straight from global memory into registers);
-// the face records with their geometry; the halo list. After the stages:
-// rho per tile and halo cell, the face slots (dh, dhu, dhv, dz) per face of
-// each tile cell, face-major, and the NS mbarriers.
+// halo's cells of U^n, the face records with their geometry, the halo list.
+// After the stages: rho per tile and halo cell (a halo cell's mu lands here
+// and is scaled in place), the halo cells' areas, the face slots
+// (dh, du, dv, dz) per face of each tile cell, face-major (placed as the
+// step's, see kSlotPad), and the NS mbarriers.
 struct AdjLayout {
   uint32_t ext, rec_cap, halo_cap;
-  uint32_t off_un, off_u1, off_lam, off_harea, off_hgn2, off_tS, off_g0, off_g1, off_g2, off_hidx;
+  uint32_t off_un, off_tS, off_g0, off_g1, off_g2, off_hidx;
   uint32_t stage;
-  uint32_t off_rho, off_slots, off_bars, total;
+  uint32_t off_rho, off_harea, off_slots, off_bars, total;
 };
 
 inline AdjLayout make_adj_layout(uint32_t w, uint32_t geo_arrays, uint32_t tc, uint32_t ns,
@@ -244,10 +301,6 @@ inline AdjLayout make_adj_layout(uint32_t w, uint32_t geo_arrays, uint32_t tc, u
   L.ext = tc + halo_cap;
   uint32_t o = 0;
   L.off_un = o; o += a16(L.ext * 4 * w);
-  L.off_u1 = o; o += a16(halo_cap * 4 * w);
-  L.off_lam = o; o += a16(halo_cap * 4 * w);
-  L.off_harea = o; o += a16(halo_cap * w);
-  L.off_hgn2 = o; o += a16(halo_cap * w);
   if (w == 4) {  // FP32: interleaved 16-byte records
     L.off_tS = o; o += a16(rec_cap * 16);
     L.off_g0 = L.off_g1 = L.off_g2 = o;
@@ -261,33 +314,68 @@ inline AdjLayout make_adj_layout(uint32_t w, uint32_t geo_arrays, uint32_t tc, u
   L.stage = o;
   o = ns * L.stage;
   L.off_rho = o; o += a16(L.ext * 4 * w);
-  L.off_slots = o; o += a16(3 * tc * 4 * w);
+  L.off_harea = o; o += a16(halo_cap * w);
+  L.off_slots = o; o += a16(3 * (tc + kSlotPad) * 4 * w);
   L.off_bars = o; o += a16(ns * 8);
   L.total = o;
   return L;
 }
 
-// Tiled adjoint of one step over the same tiles, records and work chunks as
-// k_tiled_step (scenario of each chunk, interleaved tile walk, NS-stage TMA
-// pipeline with the halo gathered by cp.async). Per tile:
-//   (A) mu and rho of every tile and halo cell (rho to shared memory, mu of
-//       the thread's own cells kept in registers);
+// Transposed friction of the last step, where the sweep starts: lambda of
+// U^{n+1} (u1) becomes mu in place (n cells), and dgn2 gets its first part.
+template <typename Real>
+__global__ void __launch_bounds__(256)
+    k_adjoint_start(const Real* u1, Real* lam, const Real* gn2, Real* dgn2, Real dt, Num num,
+                    int64_t n) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const V4<Real> c = ld4(u1 + 4 * i), l = ld4(lam + 4 * i);
+    Real mh, mx, my, b;
+    cell_vjp<Real>(c.x, c.y, c.z, l.x, l.y, l.z, gn2[i], dt, num, mh, mx, my, b);
+    st4(lam + 4 * i, mh, mx, my, l.w);
+    dgn2[i] = b;
+  }
+}
+
+// Tiled adjoint of one step over the same tiles and records as k_tiled_step
+// (interleaved tile walk, NS-stage TMA pipeline with the halo gathered by
+// cp.async), on its own chunk table. Per tile:
+//   (A) rho of every tile and halo cell in shared memory, and the staged
+//       cells (h, hu, hv, z) turned into (h, u, v, z) in place; mu of the
+//       thread's own cells stays in registers;
 //   (B) the vector-Jacobian product of every face record into the slots of
 //       the tile's cells (a face shared with another tile gives only this
 //       tile's side, as in the forward);
 //   (C) each cell: dL/dU^n = mu + its three slots in face order, the z parts
-//       added to the running dL/dz, and its dL/d(g n^2) accumulated.
+//       added to the running dL/dz; then the transposed friction of step
+//       n - 1, whose part of dL/d(g n^2) is accumulated.
 // (A) of the next tile runs right after (C), so two block barriers per tile.
+//
+// Measured per adjoint step (checkpoints at every step, 64 gauges; before:
+// lambda and U^{n+1} read by every step, friction and velocities redone for
+// halo cells and faces, gauges by one thread): FP32 1.0M cells 54.3 -> 29.2
+// us, 160,000 cells 28.0 -> 12.0, 10,000 cells 12.2 -> 9.6; FP64 (16 gauges)
+// 79,806 cells 153 -> 83, 10,000 cells 58 -> 38. FP64 is bound by the FP64
+// pipe, and by tiles not dividing over the SMs on small meshes; FP32 by
+// instruction issue and the two barriers per tile.
+//
+// Registers are capped so that 640 FP32 threads (5 blocks of 128 with
+// 256-cell tiles, which their shared memory also allows) share an SM.
+template <typename Real, int NT>
+constexpr int adjoint_min_blocks() { return (sizeof(Real) == 4 ? 640 : 256) / NT; }
+
 template <typename Real, int NT, int NS, int CPT>
-__global__ void __launch_bounds__(NT)
+__global__ void __launch_bounds__(NT, adjoint_min_blocks<Real, NT>())
     k_tiled_adjoint(DevMesh<Real> m, AdjArgs<Real> A, Num num, AdjLayout L) {
-  using O = Ops<Real>;
   constexpr int TC = NT * CPT;
+  constexpr bool kRecip = sizeof(Real) == 8;  // FP64 meshes keep 1 / area
   __shared__ int s_nrec[NS], s_nh[NS];
   extern __shared__ __align__(128) unsigned char smem[];
   Real* rho = reinterpret_cast<Real*>(smem + L.off_rho);      // [ext][4]
-  Real* slots = reinterpret_cast<Real*>(smem + L.off_slots);  // [3 TC][4]
+  Real* harea = reinterpret_cast<Real*>(smem + L.off_harea);  // [halo_cap]
+  Real* slots = reinterpret_cast<Real*>(smem + L.off_slots);  // [3 (TC + kSlotPad)][4]
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L.off_bars);
+  const Real* __restrict__ area = kRecip ? m.rarea : m.area;
 
   const Chunk ch = m.chunks[blockIdx.x];
   const int t_first = ch.tile0, n_tiles = ch.ntiles, t_step = ch.stride;
@@ -335,15 +423,12 @@ __global__ void __launch_bounds__(NT)
     }
     return ok;
   };
-  // halo cells of stage st: three interleaved cells and two scalars each
+  // halo cells of stage st: U^n into the stage, mu and area into the block's
+  // single rho and area arrays (free once the previous tile's faces are done)
   auto gather_halo = [&](int st) {
     unsigned char* p = smem + st * L.stage;
     const int32_t* hl = reinterpret_cast<const int32_t*>(p + L.off_hidx);
     Real* dun = reinterpret_cast<Real*>(p + L.off_un) + 4 * TC;
-    Real* du1 = reinterpret_cast<Real*>(p + L.off_u1);
-    Real* dla = reinterpret_cast<Real*>(p + L.off_lam);
-    Real* dar = reinterpret_cast<Real*>(p + L.off_harea);
-    Real* dgn = reinterpret_cast<Real*>(p + L.off_hgn2);
     const int nh = s_nh[st];
     constexpr int kV = 16 / (int)sizeof(Real);  // values per 16-byte copy
     for (int q = tid; q < nh; q += NT) {
@@ -351,92 +436,73 @@ __global__ void __launch_bounds__(NT)
 #pragma unroll
       for (int b = 0; b < 4 / kV; ++b) {
         cp_async16(dun + 4 * q + b * kV, A.un + 4 * c + b * kV);
-        cp_async16(du1 + 4 * q + b * kV, A.u1 + 4 * c + b * kV);
-        cp_async16(dla + 4 * q + b * kV, A.lam_in + 4 * c + b * kV);
+        cp_async16(rho + 4 * (TC + q) + b * kV, A.mu_in + 4 * c + b * kV);
       }
-      cp_async(dar + q, m.area + c);
-      cp_async(dgn + q, A.gn2 + c);
+      cp_async(harea + q, area + c);
     }
   };
 
-  // Per-cell inputs of the thread's own cells, loaded one tile ahead into
-  // registers (their latency hides behind the previous tile's face loop).
-  // load_tape_cells: U^{n+1}, g n^2 and area (tape and mesh data);
-  // load_adj_cells: lambda and dL/d(g n^2) (the previous launch's output).
-  V4<Real> nu1[CPT], nla[CPT];
-  Real ngn[CPT], nar[CPT], ndg[CPT];
-  auto load_tape_cells = [&](int t) {
+  // Per-cell inputs of the thread's own cells for (A), loaded one tile ahead
+  // into registers (their latency hides behind the previous tile's face
+  // loop): the area (mesh data) and mu (the previous launch's output).
+  V4<Real> nmu[CPT];
+  Real nar[CPT];
+  auto load_area = [&](int t) {
     const int64_t b0 = (int64_t)t * TC;
 #pragma unroll
-    for (int cc = 0; cc < CPT; ++cc) {
-      const int64_t i = b0 + tid + cc * NT;
-      nu1[cc] = ld4(A.u1 + 4 * i);
-      ngn[cc] = A.gn2[i];
-      nar[cc] = m.area[i];
-    }
+    for (int cc = 0; cc < CPT; ++cc) nar[cc] = area[b0 + tid + cc * NT];
   };
-  auto load_adj_cells = [&](int t) {
+  auto load_mu = [&](int t) {
     const int64_t b0 = (int64_t)t * TC;
 #pragma unroll
-    for (int cc = 0; cc < CPT; ++cc) {
-      const int64_t i = b0 + tid + cc * NT;
-      nla[cc] = ld4(A.lam_in + 4 * i);
-      ndg[cc] = A.dgn2[i];
-    }
+    for (int cc = 0; cc < CPT; ++cc) nmu[cc] = ld4(A.mu_in + 4 * (b0 + tid + cc * NT));
   };
-  auto load_cells = [&](int t) {
-    load_tape_cells(t);
-    load_adj_cells(t);
-  };
-  // (A) of a tile: mu (registers) and the friction and dL/dz parts of the
-  // thread's own cells from the registers load_cells filled, rho of those
-  // cells and of the halo cells this thread gathered (gather_halo's
+  auto scale = [&](Real a) { return kRecip ? -(dt * a) : -Ops<Real>::div(dt, a); };
+  // (A) of a tile: the thread's own cells from the registers load_area and
+  // load_mu filled, and the halo cells this thread gathered (gather_halo's
   // assignment, so no barrier is needed after its own copies land).
-  Real mu[CPT][3], bg[CPT], dzr[CPT];
+  V4<Real> mu[CPT];
+  Real rh[CPT];  // 1 / h of a wet cell, else 0
   auto phase_a = [&](int st, int tile) {
-    const unsigned char* p = smem + st * L.stage;
-    const Real* su1 = reinterpret_cast<const Real*>(p + L.off_u1);
-    const Real* sla = reinterpret_cast<const Real*>(p + L.off_lam);
-    const Real* har = reinterpret_cast<const Real*>(p + L.off_harea);
-    const Real* hgn = reinterpret_cast<const Real*>(p + L.off_hgn2);
+    Real* sun = reinterpret_cast<Real*>(smem + st * L.stage + L.off_un);
+    auto to_velocity = [&](Real* c) -> Real {
+      const V4<Real> x = ld4(c);
+      const Real r = Ops<Real>::wet(x.x, num) ? Ops<Real>::rcp(x.x) : Real(0);
+      st4(c, x.x, x.y * r, x.z * r, x.w);
+      return r;
+    };
     const int nc = min(TC, cell_end - tile * TC);
 #pragma unroll
     for (int cc = 0; cc < CPT; ++cc) {
       const int j = tid + cc * NT;
-      const V4<Real> c1 = nu1[cc];
-      const V4<Real> la = nla[cc];
-      dzr[cc] = la.w;
-      cell_vjp<Real>(c1.x, c1.y, c1.z, la.x, la.y, la.z, ngn[cc], dt, num, mu[cc][0], mu[cc][1],
-                     mu[cc][2], bg[cc]);
-      bg[cc] += ndg[cc];
-      const Real a = j < nc ? -O::div(dt, nar[cc]) : Real(0);  // padding: area 0
-      st4(rho + 4 * j, a * mu[cc][0], a * mu[cc][1], a * mu[cc][2], Real(0));
+      mu[cc] = nmu[cc];
+      const Real a = j < nc ? scale(nar[cc]) : Real(0);  // padding: area 0
+      st4(rho + 4 * j, a * mu[cc].x, a * mu[cc].y, a * mu[cc].z, Real(0));
+      rh[cc] = to_velocity(sun + 4 * j);
     }
     const int nh = s_nh[st];
     for (int q = tid; q < nh; q += NT) {
       const int j = TC + q;
-      const V4<Real> c1 = ld4(su1 + 4 * q);
-      const V4<Real> la = ld4(sla + 4 * q);
-      Real mh, mx, my, b;
-      cell_vjp<Real>(c1.x, c1.y, c1.z, la.x, la.y, la.z, hgn[q], dt, num, mh, mx, my, b);
-      const Real a = -O::div(dt, har[q]);
-      st4(rho + 4 * j, a * mh, a * mx, a * my, Real(0));
+      const V4<Real> c = ld4(rho + 4 * j);
+      const Real a = scale(harea[q]);
+      st4(rho + 4 * j, a * c.x, a * c.y, a * c.z, Real(0));
+      to_velocity(sun + 4 * j);
     }
   };
   int timeout = 0;
   // Programmatic dependent launch: the first tiles' tape states, records and
-  // halo lists and the own cells' tape inputs are fetched while the previous
-  // adjoint step finishes; lambda and dL/d(g n^2), its output, only after
+  // halo lists and the own cells' areas are fetched while the previous
+  // adjoint step finishes; mu and dL/d(g n^2), its output, only after
   // griddepcontrol.wait.
   if (tid == 0) {
 #pragma unroll
     for (int i = 0; i < NS - 1; ++i)
       if (i < n_tiles) issue(i, t_first + i * t_step);
   }
-  if (n_tiles > 0) load_tape_cells(t_first);
+  if (n_tiles > 0) load_area(t_first);
   pdl_trigger();
   pdl_wait();
-  if (n_tiles > 0) load_adj_cells(t_first);
+  if (n_tiles > 0) load_mu(t_first);
   if (n_tiles > 0) {
     const bool ok = (tid == 0) ? wait_stage(0) : true;
     if (__syncthreads_or(!ok)) {
@@ -456,8 +522,6 @@ __global__ void __launch_bounds__(NT)
     const int tile = t_first + k * t_step;
     const bool has_next = k + 1 < n_tiles;
     if (tid == 0 && k + NS - 1 < n_tiles) issue((k + NS - 1) % NS, tile + (NS - 1) * t_step);
-    // the next tile's own-cell inputs, into registers while the faces run
-    if (has_next) load_cells(tile + t_step);
     const unsigned char* p = smem + st * L.stage;
     const Real* sun = reinterpret_cast<const Real*>(p + L.off_un);
     const int32_t* rS = reinterpret_cast<const int32_t*>(p + L.off_tS);
@@ -467,6 +531,18 @@ __global__ void __launch_bounds__(NT)
     const int base = tile * TC;
     const int nc = min(TC, cell_end - base);
     const int nrec = s_nrec[st];
+    // what (C) and the next (A) need, into registers while the faces run
+    // (cell arrays are padded to whole tiles, so the loads are in bounds)
+    Real gn2[CPT], dg[CPT];
+#pragma unroll
+    for (int cc = 0; cc < CPT; ++cc) {
+      gn2[cc] = A.gn2[base + tid + cc * NT];
+      dg[cc] = A.dgn2[base + tid + cc * NT];
+    }
+    if (has_next) {
+      load_area(tile + t_step);
+      load_mu(tile + t_step);
+    }
 
     // (B) face records
     for (int r = tid; r < nrec; r += NT) {
@@ -486,9 +562,9 @@ __global__ void __launch_bounds__(NT)
         const int ia = (-1 - a) & (TC - 1);
         const V4<Real> UA = ld4(sun + 4 * ia);
         const V4<Real> RA = ld4(rho + 4 * ia);
-        face_vjp_clamped<Real, true>(UA, UA, nx, ny, len, num, RA.x, RA.y, RA.z, Real(0), Real(0),
-                                     Real(0), gA, gB);
-        st4(slots + 4 * (-1 - a), gA[0], gA[1], gA[2], gA[3]);
+        face_vjp<Real, true>(UA, UA, nx, ny, len, num, RA.x, RA.y, RA.z, Real(0), Real(0), Real(0),
+                             gA, gB);
+        st4(slots + 4 * slot_pad<TC>(-1 - a), gA[0], gA[1], gA[2], gA[3]);
         continue;
       }
       const int ia = a < 0 ? ((-1 - a) & (TC - 1)) : a;
@@ -497,10 +573,9 @@ __global__ void __launch_bounds__(NT)
       const V4<Real> UB = ld4(sun + 4 * ib);
       const V4<Real> RA = ld4(rho + 4 * ia);
       const V4<Real> RB = ld4(rho + 4 * ib);
-      face_vjp_clamped<Real, false>(UA, UB, nx, ny, len, num, RA.x, RA.y, RA.z, RB.x, RB.y, RB.z,
-                                    gA, gB);
-      if (a < 0) st4(slots + 4 * (-1 - a), gA[0], gA[1], gA[2], gA[3]);
-      if (b < 0) st4(slots + 4 * (-1 - b), gB[0], gB[1], gB[2], gB[3]);
+      face_vjp<Real, false>(UA, UB, nx, ny, len, num, RA.x, RA.y, RA.z, RB.x, RB.y, RB.z, gA, gB);
+      if (a < 0) st4(slots + 4 * slot_pad<TC>(-1 - a), gA[0], gA[1], gA[2], gA[3]);
+      if (b < 0) st4(slots + 4 * slot_pad<TC>(-1 - b), gB[0], gB[1], gB[2], gB[3]);
     }
     const bool ok = (tid == 0 && has_next) ? wait_stage((k + 1) % NS) : true;
     if (__syncthreads_or(!ok)) {
@@ -515,12 +590,20 @@ __global__ void __launch_bounds__(NT)
       const int j = tid + cc * NT;
       if (j >= nc) break;
       const V4<Real> f0 = ld4(slots + 4 * j);
-      const V4<Real> f1 = ld4(slots + 4 * (TC + j));
-      const V4<Real> f2 = ld4(slots + 4 * (2 * TC + j));
-      st4(A.lam_out + 4 * (int64_t)(base + j), mu[cc][0] + f0.x + f1.x + f2.x,
-          mu[cc][1] + f0.y + f1.y + f2.y, mu[cc][2] + f0.z + f1.z + f2.z,
-          dzr[cc] + f0.w + f1.w + f2.w);
-      A.dgn2[base + j] = bg[cc];
+      const V4<Real> f1 = ld4(slots + 4 * (TC + kSlotPad + j));
+      const V4<Real> f2 = ld4(slots + 4 * (2 * (TC + kSlotPad) + j));
+      const V4<Real> c = ld4(sun + 4 * j);
+      const Real su = f0.y + f1.y + f2.y, sv = f0.z + f1.z + f2.z, r = rh[cc];
+      Real lh = mu[cc].x + (f0.x + f1.x + f2.x - r * fma_rn(su, c.y, sv * c.z));
+      Real lx = fma_rn(su, r, mu[cc].y), ly = fma_rn(sv, r, mu[cc].z);
+      const Real lz = mu[cc].w + (f0.w + f1.w + f2.w);
+      if (!A.last) {
+        Real b;
+        cell_vjp<Real>(c.x, c.x * c.y, c.x * c.z, lh, lx, ly, gn2[cc], A.dt_prev, num, lh, lx, ly,
+                       b);
+        A.dgn2[base + j] = dg[cc] + b;
+      }
+      st4(A.mu_out + 4 * (int64_t)(base + j), lh, lx, ly, lz);
     }
     cp_async_wait_all();
     if (has_next) phase_a((k + 1) % NS, tile + t_step);
@@ -532,8 +615,7 @@ __global__ void __launch_bounds__(NT)
       if ((pending >> i) & 1u) mbar_wait(&bar[i], (parity_bits >> i) & 1u);
     atomicOr(A.err, kErrTimeout);
   }
-  // The last block to finish adds the gauge seeds (one thread, fixed order,
-  // so repeated gauge cells add up deterministically).
+  // The last block to finish adds the gauge seeds.
   if (A.gstep >= 0) {
     __shared__ int s_last;
     __syncthreads();
@@ -542,21 +624,18 @@ __global__ void __launch_bounds__(NT)
       s_last = atomicAdd(A.ticket, 1u) == gridDim.x - 1u;
     }
     __syncthreads();
-    if (s_last && tid == 0) {
+    if (s_last) {
       __threadfence();
-      for (int j = 0; j < A.G; ++j)
-        A.lam_out[4 * (int64_t)A.gcells[j]] += Real(A.gseed[A.gstep * A.G + j]);
-      *A.ticket = 0u;
+      add_gauge_seeds(A.mu_out, A.gauges, A.gstep, tid, NT);
+      if (tid == 0) *A.ticket = 0u;
     }
   }
 }
 
-// Adds g[k * G + j] to the depth adjoint of cell cells[j] for j < G (one
-// thread, so repeated gauge cells add up in a fixed order).
+// Adds the gauge seeds of step k to lam (one block).
 template <typename Real>
-__global__ void k_inject_gauges(Real* lam, const int32_t* cells, const double* g, int64_t k, int G) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  for (int j = 0; j < G; ++j) lam[4 * (int64_t)cells[j]] += Real(g[k * (int64_t)G + j]);
+__global__ void k_inject_gauges(Real* lam, GaugeSeeds g, long long k) {
+  add_gauge_seeds(lam, g, k, threadIdx.x, blockDim.x);
 }
 
 }  // namespace swe

@@ -18,6 +18,7 @@
 #include <algorithm>
 #include <cmath>
 #include <limits>
+#include <numeric>
 #include <vector>
 
 #include "../../include/swe.h"
@@ -203,6 +204,7 @@ struct swe_tape {
   double* gauge_dev = nullptr;
   double* gseed_dev = nullptr;
   int32_t* gcells = nullptr;
+  swe::GaugeSeeds gauges{};  // gseed_dev by distinct gauge cell
   swe::Chunk* chunks = nullptr;  // work of the adjoint kernel's blocks
   int64_t nchunks = 0;
   swe::Ctl* ctl = nullptr;      // two replay control words (one per ring)
@@ -311,7 +313,10 @@ swe_status grad_t(swe_tape* t, bool seeds_gauge, int* lam_cur) {
   cudaStream_t st = m->stream;
   int cur = 0;
   if (seeds_gauge)
-    swe::k_inject_gauges<Real><<<1, 1, 0, st>>>((Real*)t->lam[cur], t->gcells, t->gseed_dev, t->N - 1, t->G);
+    swe::k_inject_gauges<Real><<<1, 128, 0, st>>>((Real*)t->lam[cur], t->gauges, t->N - 1);
+  swe::k_adjoint_start<Real><<<grid_for(t->Tp, m->sms * 8), 256, 0, st>>>(
+      (const Real*)t->slot(t->nck - 1, t->seg_len(t->nck - 1)), (Real*)t->lam[cur], (const Real*)t->gn2,
+      (Real*)t->dgn2, Real(t->dts[t->N - 1]), num_of(m), t->Tp);
   // Replays run one segment ahead on the side stream: segment seg - 1's
   // replay (ring (seg - 1) % 2) overlaps segment seg's adjoint steps; it
   // first waits for the adjoint of segment seg + 1, the ring's last user.
@@ -330,16 +335,15 @@ swe_status grad_t(swe_tape* t, bool seeds_gauge, int* lam_cur) {
       const int64_t r = j - j0;
       swe::AdjArgs<Real> a{};
       a.un = (const Real*)t->slot(seg, r);
-      a.u1 = (const Real*)t->slot(seg, r + 1);
-      a.lam_in = (const Real*)t->lam[cur];
-      a.lam_out = (Real*)t->lam[cur ^ 1];
+      a.mu_in = (const Real*)t->lam[cur];
+      a.mu_out = (Real*)t->lam[cur ^ 1];
       a.gn2 = (const Real*)t->gn2;
       a.dgn2 = (Real*)t->dgn2;
       a.dt = Real(t->dts[j]);
+      a.dt_prev = j > 0 ? Real(t->dts[j - 1]) : Real(0);
+      a.last = j == 0;
       a.err = t->err;
-      a.gcells = t->gcells;
-      a.gseed = t->gseed_dev;
-      a.G = t->G;
+      a.gauges = t->gauges;
       a.gstep = (seeds_gauge && j >= 1) ? (long long)(j - 1) : -1ll;  // lambda^j gets dL/dh^j
       a.ticket = t->ticket;
       launch_adjoint<Real>(m, t->chunks, (int)t->nchunks, a, t->adj, st);
@@ -390,13 +394,14 @@ swe_status grad_record(swe_state* s, int64_t n_steps, int64_t checkpoint_every,
     free_tape(t);
     return SWE_ECUDA;
   }
-  // adjoint chunk table: one wave of resident blocks over the scenario's tiles
+  // Adjoint chunk table: one wave of resident blocks, one chunk for every
+  // block slot (chunks of equal tile counts leave slots empty: 313 FP64 tiles
+  // on 304 slots made 157 chunks of 2, some SMs with 4 tiles and others with 2).
   std::vector<swe::Chunk> chunks;
   {
     const Scenario& sc = m->scen[0];
     const int64_t resident = (int64_t)m->sms * occ;
-    const int64_t per = std::max<int64_t>(1, (sc.ntiles + resident - 1) / resident);
-    const int64_t nc = (sc.ntiles + per - 1) / per;
+    const int64_t nc = std::min<int64_t>(sc.ntiles, resident);
     for (int64_t r = 0; r < nc; ++r) {
       swe::Chunk c{};
       c.scen = 0;
@@ -424,6 +429,7 @@ swe_status grad_record(swe_state* s, int64_t n_steps, int64_t checkpoint_every,
   L.add(8 * t->N * std::max(1, t->G));  // gauge depths
   L.add(8 * t->N * std::max(1, t->G));  // gauge seeds
   L.add(4 * std::max(1, t->G));
+  L.add(4 * (3 * (size_t)t->G + 1));  // gauges by cell
   L.add(sizeof(swe::Chunk) * chunks.size());
   L.add(2 * sizeof(swe::Ctl));
   L.add(2 * 8 * (size_t)std::max<int64_t>(1, m->nchunks));
@@ -449,6 +455,7 @@ swe_status grad_record(swe_state* s, int64_t n_steps, int64_t checkpoint_every,
   t->gauge_dev = (double*)t->arena.take(8 * t->N * std::max(1, t->G));
   t->gseed_dev = (double*)t->arena.take(8 * t->N * std::max(1, t->G));
   t->gcells = (int32_t*)t->arena.take(4 * std::max(1, t->G));
+  int32_t* by_cell = (int32_t*)t->arena.take(4 * (3 * (size_t)t->G + 1));
   t->chunks = (swe::Chunk*)t->arena.take(sizeof(swe::Chunk) * chunks.size());
   t->ctl = (swe::Ctl*)t->arena.take(2 * sizeof(swe::Ctl));
   t->partial = (double*)t->arena.take(2 * 8 * (size_t)std::max<int64_t>(1, m->nchunks));
@@ -481,7 +488,24 @@ swe_status grad_record(swe_state* s, int64_t n_steps, int64_t checkpoint_every,
     for (int64_t j = 0; j < m->Tp; ++j)
       if (perm[j] >= 0) inv[perm[j]] = (int32_t)j;
     for (int j = 0; j < t->G; ++j) gi[j] = inv[gauge_cells[j]];
-    if (cuda_failed(cudaMemcpyAsync(t->gcells, gi.data(), 4 * t->G, cudaMemcpyHostToDevice, m->stream)) ||
+    // the distinct cells, and each one's gauges in ascending order
+    std::vector<int32_t> cells, first, index(t->G);
+    std::iota(index.begin(), index.end(), 0);
+    std::stable_sort(index.begin(), index.end(), [&](int32_t a, int32_t b) { return gi[a] < gi[b]; });
+    for (int q = 0; q < t->G; ++q)
+      if (q == 0 || gi[index[q]] != cells.back()) {
+        cells.push_back(gi[index[q]]);
+        first.push_back(q);
+      }
+    first.push_back(t->G);
+    const int nc = (int)cells.size();
+    t->gauges = {by_cell, by_cell + t->G, by_cell + 2 * t->G + 1, t->gseed_dev, t->G, nc};
+    auto put = [&](const int32_t* to, const std::vector<int32_t>& v) {
+      return cuda_failed(cudaMemcpyAsync((void*)to, v.data(), 4 * v.size(), cudaMemcpyHostToDevice,
+                                         m->stream));
+    };
+    if (put(t->gauges.cells, cells) || put(t->gauges.first, first) || put(t->gauges.index, index) ||
+        put(t->gcells, gi) ||
         cuda_failed(cudaStreamSynchronize(m->stream)))
       return fail(SWE_ECUDA);
   }
@@ -531,7 +555,6 @@ swe_status grad(swe_tape* t, const double* g_h, const double* g_hu, const double
   const cudaMemcpyKind in_kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
   CK(cudaMemsetAsync(t->lam[0], 0, sb, st));
   CK(cudaMemsetAsync(t->lam[1], 0, sb, st));
-  CK(cudaMemsetAsync(t->dgn2, 0, t->w * t->Tp, st));
   CK(cudaMemsetAsync(t->err, 0, sizeof(int), st));
   CK(cudaMemsetAsync(t->ticket, 0, sizeof(unsigned int), st));
   const double* seeds[3] = {g_h, g_hu, g_hv};

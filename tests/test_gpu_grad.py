@@ -333,3 +333,23 @@ def test_fp32_calibration_gradient_when_misfits_exceed_fp32_resolution():
         den = np.abs(ref).max()
         assert np.abs(res["f32"]["grad"][k] - ref).max() <= 1e-4 * den, k
         assert np.abs(seeded[k] - ref).max() <= 2e-5 * den, k
+
+
+@pytest.mark.parametrize("n_steps,tile", [(1, 256), (5, 64), (5, 256), (4, 512)])
+def test_adjoint_with_many_repeated_gauges_and_frictionless_cells(n_steps, tile):
+    """More gauges than a block has threads, several in one cell (their seeds
+    add up by cell), and cells without friction (their transposed friction is
+    skipped), on a mesh of one full tile and a partial one (larger tiles: a
+    partial one): the dot-product test, 1e-10 relative."""
+    c = smooth_wet_case(nx=16, ny=9, seed=21)
+    c.n[::3] = 0.0
+    rng = np.random.default_rng(8)
+    gauges = rng.integers(0, c.mesh.n_tris, size=300).tolist()
+    mesh, st, tape = record(c, n_steps, 2, gauges, tile=tile)
+    g = seeds(c, n_steps, len(gauges), 22)
+    grads = tape.grad(**g)
+    for which in ("h", "z", "n", "all"):
+        v = directions(c, 23, which)
+        t, gd, _ = oracle_jvp(c, n_steps, gauges, v)
+        lhs, rhs = pair(g, v, t, gd, grads)
+        assert abs(lhs - rhs) <= 1e-10 * max(abs(lhs), 1e-300), (which, lhs, rhs)
