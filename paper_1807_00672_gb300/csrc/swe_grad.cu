@@ -3,18 +3,25 @@
 // swe_grad_record runs n steps forward on a state, as swe_run does, and
 // keeps a tape: the dt of every step (held fixed for the derivative), the
 // depths at the gauge cells after every step, and the state every K steps
-// (checkpoints). swe_grad then runs the adjoint backwards through the steps:
-// segment by segment, from the last checkpoint to the first, it recomputes
-// the segment's inner states from its checkpoint with the forward kernel
-// (the forward is deterministic, so the replay reproduces the recorded
-// states bit for bit; the replay's dt is checked against the recorded one;
-// the segment's last state is the next checkpoint, or the final state, and
-// is not recomputed) and applies the tiled adjoint kernel step by step,
-// adding the gauge-loss seeds as it passes their steps. The replay of the
-// next segment runs on a second stream while the current segment's adjoint
-// steps run, each into its own ring of states. Memory: ceil(n / K) + 1
-// checkpoints, 2 (K - 1) replayed states and two adjoint states. K = 1
-// keeps every state and replays nothing.
+// (checkpoints). The recorded steps write straight into the tape's buffers,
+// the way a replay does: a segment's inner states into one of two rings (the
+// last segment's into a buffer of their own), its end into the next
+// checkpoint; the steps follow each other without copies or other launches
+// between them (1.0M FP32 cells, K = 50: 27.1 us per recorded step when each
+// was followed by a launch that noted its dt and gauges, and the last
+// segment's by a copy; 21.3 now). swe_grad then runs the adjoint backwards
+// through the steps: segment by segment, from the last checkpoint to the
+// first. The inner states of the last three segments are still there from
+// the recording; those of an earlier one are recomputed from its checkpoint
+// with the forward kernel (the forward is deterministic, so the replay
+// reproduces the recorded states bit for bit; the replay's dt is checked
+// against the recorded one; the segment's last state is the next checkpoint,
+// or the final state, and is not recomputed). The tiled adjoint kernel runs
+// step by step, adding the gauge-loss seeds as it passes their steps. The
+// replay of the next segment runs on a second stream while the current
+// segment's adjoint steps run, each into its own ring of states. Memory:
+// ceil(n / K) + 1 checkpoints, up to 3 (K - 1) inner states and two adjoint
+// states. K = 1 keeps every state and replays nothing.
 #include <algorithm>
 #include <cmath>
 #include <limits>
@@ -39,26 +46,63 @@ namespace {
 
 constexpr int kErrReplay = 8;  // a replayed step did not reproduce the recorded dt
 
-// After forward step k: its dt and the gauge depths of the new state.
+// States of a tape, sb bytes each: checkpoint seg (U^{seg K}) at ck + seg sb,
+// U^N behind the last one. Inner states U^{seg K + 1} .. of segment seg lie in
+// ring seg % 2, so that the replay of the next segment (on the side stream)
+// overlaps the adjoint steps of the current one, those of the last segment in
+// `tail`.
+struct TapeSlots {
+  char *ck, *ring[2], *tail;
+  int64_t N, K, nck;
+  size_t sb;
+  __host__ __device__ int64_t seg_len(int64_t seg) const {
+    return (seg + 1) * K < N ? K : N - seg * K;
+  }
+  __host__ __device__ char* slot(int64_t seg, int64_t r) const {  // state U^{seg K + r}
+    if (r == 0) return ck + seg * sb;
+    if (r == seg_len(seg)) return ck + (seg + 1) * sb;
+    if (seg == nck - 1) return tail + (r - 1) * sb;
+    return ring[seg % 2] + (r - 1) * sb;
+  }
+  __host__ __device__ char* state(int64_t n) const {  // U^n
+    if (n == 0) return ck;
+    const int64_t seg = (n - 1) / K;
+    return slot(seg, n - seg * K);
+  }
+};
+
+// Gauge depths after steps k0 .. k1 - 1.
 template <typename Real>
-__global__ void k_record_step(const swe::Ctl* ctl, const Real* b0, const Real* b1, double* dts,
-                              int64_t k, const int32_t* cells, int G, double* gauge) {
-  const Real* U = ctl->cur ? b1 : b0;
-  if (blockIdx.x == 0 && threadIdx.x == 0) dts[k] = ctl->dt_last;
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < G; j += gridDim.x * blockDim.x)
-    gauge[k * (int64_t)G + j] = (double)U[4 * (int64_t)cells[j]];
+__global__ void __launch_bounds__(128)
+    k_tape_gauges(TapeSlots s, int64_t k0, int64_t k1, const int32_t* cells, int G, double* gauge) {
+  for (int64_t i = k0 * G + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < k1 * G;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t k = i / G;
+    gauge[i] = (double)((const Real*)s.state(k + 1))[4 * (int64_t)cells[i - k * G]];
+  }
 }
 
-// Copies the current buffer (n interleaved cells) to dst.
+// n interleaved cells: the state's current buffer to the tape's U^0, or the
+// tape's newest state (steps0: the state's steps before the recording) back.
 template <typename Real>
-__global__ void k_copy_current(const swe::Ctl* ctl, const Real* b0, const Real* b1, Real* dst,
-                               int64_t n) {
-  const Real* U = ctl->cur ? b1 : b0;
+__global__ void __launch_bounds__(256)
+    k_copy_state(const swe::Ctl* ctl, Real* b0, Real* b1, TapeSlots s, long long steps0, int to_tape,
+                 int64_t n) {
+  Real* own = ctl->cur ? b1 : b0;
+  Real* tape = (Real*)s.state(to_tape ? 0 : ctl->steps - steps0);
+  const Real* from = to_tape ? own : tape;
+  Real* to = to_tape ? tape : own;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const swe::V4<Real> v = swe::ld4(U + 4 * i);
-    swe::st4(dst + 4 * i, v.x, v.y, v.z, v.w);
+    const swe::V4<Real> v = swe::ld4(from + 4 * i);
+    swe::st4(to + 4 * i, v.x, v.y, v.z, v.w);
   }
+}
+
+// Caller cells -> internal cells, in place.
+__global__ void k_internal_cells(const int32_t* iperm, int32_t* cells, int n) {
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x)
+    cells[j] = iperm[cells[j]];
 }
 
 // Replay control word: buffer 0 current, the recorded dt, no end time.
@@ -185,14 +229,10 @@ struct swe_tape {
   size_t w = 8;
   int64_t Tp = 0, T = 0;
   Arena arena;
-  char* ck = nullptr;    // nck + 1 states of Tp interleaved cells: U^0, U^K, U^2K, ..., U^N
-  // Two rings of K - 1 replayed states U^{j0+1} .. U^{j0+K-1}: segment seg
-  // uses ring seg % 2, so the replay of the next segment (on the side
-  // stream) overlaps the adjoint steps of the current one. The last
-  // segment's inner states are kept from the recording in `tail`, so a
-  // backward sweep starts with adjoint steps instead of a replay.
-  char* ring[2] = {nullptr, nullptr};
-  char* tail = nullptr;
+  TapeSlots slots{};
+  // The segment whose inner states each ring holds (-1: none): the recording
+  // leaves the last but one and two there, a replay the one it recomputed.
+  int64_t holds[2] = {-1, -1};
   cudaStream_t side = nullptr;
   cudaEvent_t replayed[2] = {nullptr, nullptr}, consumed[2] = {nullptr, nullptr};
   char* lam[2] = {nullptr, nullptr};
@@ -217,13 +257,8 @@ struct swe_tape {
   cudaEvent_t ev[2] = {nullptr, nullptr};
 
   size_t state_bytes() const { return 4 * w * (size_t)Tp; }
-  int64_t seg_len(int64_t seg) const { return std::min(N, (seg + 1) * K) - seg * K; }
-  void* slot(int64_t seg, int64_t r) const {  // state U^{seg K + r} of segment seg
-    if (r == 0) return ck + seg * state_bytes();
-    if (r == seg_len(seg)) return ck + (seg + 1) * state_bytes();
-    if (seg == nck - 1) return tail + (r - 1) * state_bytes();
-    return ring[seg % 2] + (r - 1) * state_bytes();
-  }
+  int64_t seg_len(int64_t seg) const { return slots.seg_len(seg); }
+  void* slot(int64_t seg, int64_t r) const { return slots.slot(seg, r); }
 };
 
 namespace {
@@ -244,19 +279,28 @@ void free_tape(swe_tape* t) {
   if (m) release_mesh(m);
 }
 
-// Device state view of replay step r of segment seg (input slot r, output
-// slot r + 1; the current buffer alternates as the replay control word says).
+// Step r of segment seg on the tape's buffers: the current buffer (number
+// cur when r is even) is its input slot, the other one its output slot.
+template <typename Real>
+void set_buffers(const swe_tape* t, int64_t seg, int64_t r, int cur, swe::DevState<Real>& d) {
+  Real* in = (Real*)t->slot(seg, r);
+  Real* out = (Real*)t->slot(seg, r + 1);
+  for (int b = 0; b < 2; ++b) {
+    Real* p = b == cur ? in : out;
+    d.h[b] = p;
+    d.hu[b] = p + 1;
+    d.hv[b] = p + 2;
+  }
+  d.stride = 4;
+  d.z = in + 3;
+}
+
+// Device state view of replay step r of segment seg (the replay control word
+// starts with buffer 0 current).
 template <typename Real>
 swe::DevState<Real> replay_state(const swe_tape* t, int64_t seg, int64_t r) {
   swe::DevState<Real> d{};
-  Real* in = (Real*)t->slot(seg, r);
-  Real* out = (Real*)t->slot(seg, r + 1);
-  Real* b0 = (r % 2 == 0) ? in : out;
-  Real* b1 = (r % 2 == 0) ? out : in;
-  d.h[0] = b0; d.hu[0] = b0 + 1; d.hv[0] = b0 + 2;
-  d.h[1] = b1; d.hu[1] = b1 + 1; d.hv[1] = b1 + 2;
-  d.stride = 4;
-  d.z = b0 + 3;
+  set_buffers(t, seg, r, (int)(r % 2), d);
   d.gn2 = (const Real*)t->gn2;
   d.partial = t->partial + (seg % 2) * std::max<int64_t>(1, t->mesh->nchunks);
   d.ctl = t->ctl + seg % 2;
@@ -268,28 +312,38 @@ swe_status record_t(swe_state* s, swe_tape* t) {
   swe_mesh* m = s->mesh;
   cudaStream_t st = m->stream;
   const int gs = grid_for(t->Tp, m->sms * 8);
-  const Real* b0 = (const Real*)s->h[0];
-  const Real* b1 = (const Real*)s->h[1];
-  k_copy_current<Real><<<gs, 256, 0, st>>>(s->ctl, b0, b1, (Real*)t->ck, t->Tp);
+  Real* b0 = (Real*)s->h[0];
+  Real* b1 = (Real*)s->h[1];
+  const long long steps0 = s->host_ctl[0].steps;
+  const int cur0 = s->host_ctl[0].cur;
+  k_copy_state<Real><<<gs, 256, 0, st>>>(s->ctl, b0, b1, t->slots, steps0, 1, t->Tp);
   CK(cudaMemcpyAsync(t->gn2, s->gn2, t->w * t->Tp, cudaMemcpyDeviceToDevice, st));
   CK(cudaEventRecord(t->ev[0], st));
-  const int64_t j_tail = (t->nck - 1) * t->K;  // first step of the last segment
+  auto gauges = [&](int64_t k0, int64_t k1) {
+    if (t->G > 0)
+      k_tape_gauges<Real><<<(int)std::min<int64_t>(((k1 - k0) * t->G + 127) / 128, m->sms * 8), 128, 0,
+                            st>>>(t->slots, k0, k1, t->gcells, t->G, t->gauge_dev);
+  };
+  int64_t noted = 0;  // steps whose gauges are taken
   for (int64_t k = 0; k < t->N; ++k) {
-    launch_forward(m, dev_state<Real>(s), st);
-    k_record_step<Real><<<1, 128, 0, st>>>(s->ctl, b0, b1, t->dts_dev, k, t->gcells, t->G,
-                                           t->gauge_dev);
-    if (k + 1 > j_tail && k + 1 < t->N)  // an inner state of the last segment
-      k_copy_current<Real><<<gs, 256, 0, st>>>(s->ctl, b0, b1,
-                                               (Real*)t->slot(t->nck - 1, k + 1 - j_tail), t->Tp);
-    if ((k + 1) % t->K == 0 || k + 1 == t->N)
-      k_copy_current<Real><<<gs, 256, 0, st>>>(s->ctl, b0, b1,
-                                               (Real*)(t->ck + ((k + t->K) / t->K) * t->state_bytes()),
-                                               t->Tp);
+    const int64_t seg = k / t->K;
+    // a ring is about to be used again: take the gauges of the steps so far
+    if (k == seg * t->K && t->K > 1 && seg >= 2 && seg < t->nck - 1) {
+      gauges(noted, k);
+      noted = k;
+    }
+    swe::DevState<Real> d = dev_state<Real>(s);
+    set_buffers(t, seg, k - seg * t->K, (int)((cur0 + k) % 2), d);
+    d.dt_log = t->dts_dev + k;
+    launch_forward(m, d, st);
   }
+  gauges(noted, t->N);
+  k_copy_state<Real><<<gs, 256, 0, st>>>(s->ctl, b0, b1, t->slots, steps0, 0, t->Tp);
   CK(cudaEventRecord(t->ev[1], st));
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(st));
   CK(cudaEventElapsedTime(&t->record_ms, t->ev[0], t->ev[1]));
+  for (int64_t seg = std::max<int64_t>(0, t->nck - 3); seg < t->nck - 1; ++seg) t->holds[seg % 2] = seg;
   return SWE_OK;
 }
 
@@ -320,15 +374,17 @@ swe_status grad_t(swe_tape* t, bool seeds_gauge, int* lam_cur) {
   // Replays run one segment ahead on the side stream: segment seg - 1's
   // replay (ring (seg - 1) % 2) overlaps segment seg's adjoint steps; it
   // first waits for the adjoint of segment seg + 1, the ring's last user.
-  // The last segment needs none (its states are in the tail).
+  // The last segment needs none (its states are in the tail), nor does one
+  // whose states its ring still holds.
   CK(cudaEventRecord(t->consumed[0], st));
   CK(cudaEventRecord(t->consumed[1], st));
   for (int64_t seg = t->nck - 1; seg >= 0; --seg) {
     const int64_t j0 = seg * t->K, j1 = std::min(t->N, j0 + t->K);
-    if (seg >= 1) {
+    if (seg >= 1 && t->holds[(seg - 1) % 2] != seg - 1) {
       CK(cudaStreamWaitEvent(t->side, t->consumed[(seg - 1) % 2], 0));
       replay_segment<Real>(t, seg - 1, t->side);
       CK(cudaEventRecord(t->replayed[(seg - 1) % 2], t->side));
+      t->holds[(seg - 1) % 2] = seg - 1;
     }
     if (seg < t->nck - 1) CK(cudaStreamWaitEvent(st, t->replayed[seg % 2], 0));
     for (int64_t j = j1 - 1; j >= j0; --j) {
@@ -416,10 +472,10 @@ swe_status grad_record(swe_state* s, int64_t n_steps, int64_t checkpoint_every,
   }
   const size_t sb = t->state_bytes();
   Layout L;
+  const size_t inner = sb * (size_t)(t->K - 1);  // a segment's inner states
+  const int rings = (int)std::min<int64_t>(2, t->nck - 1);
   L.add(sb * (t->nck + 1));
-  L.add(sb * std::max<int64_t>(1, t->K - 1));
-  L.add(sb * std::max<int64_t>(1, t->K - 1));
-  L.add(sb * std::max<int64_t>(1, t->K - 1));  // tail
+  for (int i = 0; i <= rings; ++i) L.add(inner);  // the rings and the tail
   L.add(sb); L.add(sb);
   L.add(t->w * t->Tp);  // gn2
   L.add(t->w * t->Tp);  // dgn2
@@ -441,10 +497,13 @@ swe_status grad_record(swe_state* s, int64_t n_steps, int64_t checkpoint_every,
     return SWE_ENOMEM;
   }
   t->arena.size = L.total;
-  t->ck = (char*)t->arena.take(sb * (t->nck + 1));
-  t->ring[0] = (char*)t->arena.take(sb * std::max<int64_t>(1, t->K - 1));
-  t->ring[1] = (char*)t->arena.take(sb * std::max<int64_t>(1, t->K - 1));
-  t->tail = (char*)t->arena.take(sb * std::max<int64_t>(1, t->K - 1));
+  t->slots.N = t->N;
+  t->slots.K = t->K;
+  t->slots.nck = t->nck;
+  t->slots.sb = sb;
+  t->slots.ck = (char*)t->arena.take(sb * (t->nck + 1));
+  for (int i = 0; i < rings; ++i) t->slots.ring[i] = (char*)t->arena.take(inner);
+  t->slots.tail = (char*)t->arena.take(inner);
   t->lam[0] = (char*)t->arena.take(sb);
   t->lam[1] = (char*)t->arena.take(sb);
   t->gn2 = t->arena.take(t->w * t->Tp);
@@ -467,7 +526,17 @@ swe_status grad_record(swe_state* s, int64_t n_steps, int64_t checkpoint_every,
     return SWE_ECUDA;
   }
   auto fail = [&](swe_status r) { free_tape(t); return r; };
-  if (cuda_failed(cudaMemsetAsync(t->arena.base, 0, L.total, m->stream)) ||
+  // The steps write every cell of a state; its padding (read by copies of
+  // whole tiles, never used) is set once.
+  auto zero_padding = [&](char* states, int64_t n) {
+    const size_t used = 4 * t->w * (size_t)t->T;
+    return n > 0 && sb > used &&
+           cuda_failed(cudaMemset2DAsync(states + used, sb, 0, sb - used, (size_t)n, m->stream));
+  };
+  if (zero_padding(t->slots.ck, t->nck + 1) || zero_padding(t->slots.tail, t->K - 1) ||
+      (rings > 0 && zero_padding(t->slots.ring[0], t->K - 1)) ||
+      (rings > 1 && zero_padding(t->slots.ring[1], t->K - 1)) ||
+      cuda_failed(cudaMemsetAsync(t->lam[0], 0, t->arena.base + L.total - t->lam[0], m->stream)) ||
       cuda_failed(cudaEventCreate(&t->ev[0])) || cuda_failed(cudaEventCreate(&t->ev[1])) ||
       cuda_failed(cudaStreamCreateWithFlags(&t->side, cudaStreamNonBlocking)))
     return fail(SWE_ECUDA);
@@ -481,13 +550,13 @@ swe_status grad_record(swe_state* s, int64_t n_steps, int64_t checkpoint_every,
     return fail(SWE_ECUDA);
   // gauge cells in internal order
   if (t->G > 0) {
-    std::vector<int32_t> perm(m->Tp), inv(m->T, -1), gi(t->G);
-    if (cuda_failed(cudaMemcpyAsync(perm.data(), m->perm, 4 * m->Tp, cudaMemcpyDeviceToHost, m->stream)) ||
+    std::vector<int32_t> gi(t->G);
+    if (cuda_failed(cudaMemcpyAsync(t->gcells, gauge_cells, 4 * t->G, cudaMemcpyHostToDevice, m->stream)))
+      return fail(SWE_ECUDA);
+    k_internal_cells<<<grid_for(t->G, m->sms), 256, 0, m->stream>>>(m->iperm, t->gcells, t->G);
+    if (cuda_failed(cudaMemcpyAsync(gi.data(), t->gcells, 4 * t->G, cudaMemcpyDeviceToHost, m->stream)) ||
         cuda_failed(cudaStreamSynchronize(m->stream)))
       return fail(SWE_ECUDA);
-    for (int64_t j = 0; j < m->Tp; ++j)
-      if (perm[j] >= 0) inv[perm[j]] = (int32_t)j;
-    for (int j = 0; j < t->G; ++j) gi[j] = inv[gauge_cells[j]];
     // the distinct cells, and each one's gauges in ascending order
     std::vector<int32_t> cells, first, index(t->G);
     std::iota(index.begin(), index.end(), 0);
@@ -505,7 +574,6 @@ swe_status grad_record(swe_state* s, int64_t n_steps, int64_t checkpoint_every,
                                          m->stream));
     };
     if (put(t->gauges.cells, cells) || put(t->gauges.first, first) || put(t->gauges.index, index) ||
-        put(t->gcells, gi) ||
         cuda_failed(cudaStreamSynchronize(m->stream)))
       return fail(SWE_ECUDA);
   }
@@ -606,6 +674,7 @@ swe_status grad(swe_tape* t, const double* g_h, const double* g_hu, const double
   CK(cudaStreamSynchronize(st));
   CK(cudaGetLastError());
   CK(cudaEventElapsedTime(&t->grad_ms, t->ev[0], t->ev[1]));
+  if (err) t->holds[0] = t->holds[1] = -1;  // no ring to rely on
   if (err & swe::kErrTimeout) return SWE_ETIMEOUT;
   if (err) return SWE_ESTATE;  // the replay did not reproduce the recorded steps
   return SWE_OK;

@@ -353,3 +353,34 @@ def test_adjoint_with_many_repeated_gauges_and_frictionless_cells(n_steps, tile)
         t, gd, _ = oracle_jvp(c, n_steps, gauges, v)
         lhs, rhs = pair(g, v, t, gd, grads)
         assert abs(lhs - rhs) <= 1e-10 * max(abs(lhs), 1e-300), (which, lhs, rhs)
+
+
+@pytest.mark.parametrize("n_steps,K", [(3, 4), (4, 2), (9, 3), (10, 3), (13, 3), (11, 2), (5, 1)])
+def test_recorded_segments_and_a_second_sweep(n_steps, K):
+    """From one segment to six: segments whose inner states the recording
+    left in place, recomputed ones, a partial last one. The gauge depths, the
+    time and the final state equal plain steps bitwise, and a second sweep
+    over the same tape (whose first replays overwrote what the recording
+    left) gives the same bits as the first and as a tape that keeps every
+    state."""
+    c = smooth_wet_case(nx=20, ny=11, seed=31)
+    gauges = [0, 17, c.mesh.n_tris - 1]
+    mesh, st, tape = record(c, n_steps, K, gauges, tile=64)
+    plain = swe.State(mesh, c.h, c.hu, c.hv, c.z, c.n)
+    gh = np.zeros((n_steps, 3))
+    for k in range(n_steps):
+        plain.step()
+        gh[k] = plain.fields()[0][gauges]
+    assert np.array_equal(tape.gauge_h, gh)
+    assert st.t == plain.t
+    for a, b in zip(st.fields(), plain.fields()):
+        assert np.array_equal(a, b)
+    g = seeds(c, n_steps, 3, 32)
+    first, second = tape.grad(**g), tape.grad(**g)
+    _, _, every = record(c, n_steps, 1, gauges, tile=64)
+    ref = every.grad(**g)
+    for k in ref:
+        assert np.array_equal(first[k], ref[k]) and np.array_equal(second[k], ref[k]), k
+    st.step()  # the state goes on from where the recording ended
+    plain.step()
+    assert np.array_equal(st.fields()[0], plain.fields()[0])
