@@ -15,6 +15,7 @@
 #include <cstdio>
 #include <cstring>
 #include <limits>
+#include <mutex>
 #include <string>
 #include <thread>
 #include <type_traits>
@@ -150,6 +151,118 @@ bool cuda_failed_at(cudaError_t e, const char* what, const char* file, int line)
   g_cuda_msg = std::string(cudaGetErrorString(e)) + " in " + what + " (" + base + ":" +
                std::to_string(line) + ")";
   return true;
+}
+
+namespace {
+
+constexpr size_t kKeptBytes = size_t(2) << 30;  // most bytes kept per device
+
+struct KeptArena {
+  int device;
+  char* base;
+  size_t bytes;
+};
+std::mutex g_kept_mutex;
+std::vector<KeptArena> g_kept;  // oldest first
+int g_live_meshes = 0;
+
+// Gives back kept arenas, oldest first, until `device` keeps at most `most`
+// bytes (device -1: all arenas of every device).
+void drop_kept(int device, size_t most) noexcept {
+  for (;;) {
+    char* base = nullptr;
+    {
+      std::lock_guard<std::mutex> lock(g_kept_mutex);
+      size_t sum = 0;
+      for (const KeptArena& k : g_kept)
+        if (device < 0 || k.device == device) sum += k.bytes;
+      if (sum <= most) return;
+      for (size_t i = 0; !base; ++i)
+        if (device < 0 || g_kept[i].device == device) {
+          base = g_kept[i].base;
+          g_kept.erase(g_kept.begin() + (std::ptrdiff_t)i);
+        }
+    }
+    cudaFree(base);
+  }
+}
+
+}  // namespace
+
+cudaError_t device_alloc(char** p, size_t bytes) {
+  cudaError_t e = cudaMalloc((void**)p, bytes);
+  int dev = 0;
+  if (e != cudaSuccess && cudaGetDevice(&dev) == cudaSuccess) {
+    cudaGetLastError();
+    drop_kept(dev, 0);
+    e = cudaMalloc((void**)p, bytes);
+  }
+  if (e != cudaSuccess) *p = nullptr;
+  return e;
+}
+
+bool arena_alloc(Arena& a, size_t bytes) {
+  a = Arena();
+  if (cudaGetDevice(&a.device) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  {
+    std::lock_guard<std::mutex> lock(g_kept_mutex);
+    size_t best = g_kept.size();
+    for (size_t i = 0; i < g_kept.size(); ++i)  // the tightest that wastes at most half of itself
+      if (g_kept[i].device == a.device && g_kept[i].bytes >= bytes && g_kept[i].bytes / 2 <= bytes &&
+          (best == g_kept.size() || g_kept[i].bytes < g_kept[best].bytes))
+        best = i;
+    if (best < g_kept.size()) {
+      a.base = g_kept[best].base;
+      a.held = g_kept[best].bytes;
+      g_kept.erase(g_kept.begin() + (std::ptrdiff_t)best);
+    }
+  }
+  if (!a.base) {
+    if (device_alloc(&a.base, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    a.held = bytes;
+  }
+  a.size = bytes;
+  return true;
+}
+
+void arena_free(Arena& a) noexcept {
+  if (!a.base) return;
+  bool keep = a.held <= kKeptBytes;
+  if (keep && a.held > kKeptBytes / 32) {  // a large one only while the device has room
+    int dev = -1;
+    size_t room = 0, total = 0;
+    keep = cudaGetDevice(&dev) == cudaSuccess && dev == a.device &&
+           cudaMemGetInfo(&room, &total) == cudaSuccess && room > total / 2;
+  }
+  if (keep) {
+    try {
+      std::lock_guard<std::mutex> lock(g_kept_mutex);
+      g_kept.push_back({a.device, a.base, a.held});
+    } catch (...) {
+      keep = false;
+    }
+  }
+  if (keep) drop_kept(a.device, kKeptBytes);
+  else cudaFree(a.base);
+  a = Arena();
+}
+
+// Meshes of the process that are alive: the last to go takes the kept arenas
+// along.
+void count_mesh(int d) noexcept {
+  bool last;
+  {
+    std::lock_guard<std::mutex> lock(g_kept_mutex);
+    g_live_meshes += d;
+    last = g_live_meshes == 0;
+  }
+  if (last) drop_kept(-1, 0);
 }
 
 }  // namespace swe_host
@@ -845,12 +958,12 @@ swe_status create_batch(int32_t n, const double* const* xy, const int64_t* n_nod
   }
   const size_t bare = L.total;
   if (m->res.nblocks > 0) L.add(m->res.blob.size());
-  cudaError_t got = cudaMalloc((void**)&m->arena.base, L.total);
+  cudaError_t got = device_alloc(&m->arena.base, L.total);
   if (got != cudaSuccess && m->res.nblocks > 0) {  // without the resident kernel's parts
     cudaGetLastError();
     m->res = ResidentMesh();
     L.total = bare;
-    got = cudaMalloc((void**)&m->arena.base, L.total);
+    got = device_alloc(&m->arena.base, L.total);
   }
   if (got != cudaSuccess) {
     cudaGetLastError();
@@ -1052,6 +1165,8 @@ swe_status create_batch(int32_t n, const double* const* xy, const int64_t* n_nod
     swe_mesh_destroy(m);
     return st;
   }
+  m->counted = true;
+  count_mesh(1);
   *out = m;
   return SWE_OK;
 }
@@ -1083,6 +1198,7 @@ swe_status read_ctl(const swe_state* s) {
 
 static void free_mesh(swe_mesh* m) {
   if (m->arena.base) cudaFree(m->arena.base);
+  if (m->counted) count_mesh(-1);
   if (m->own_stream && m->stream) cudaStreamDestroy(m->stream);
   delete m;
 }
@@ -1266,12 +1382,10 @@ swe_status state_init(swe_mesh* m, const double* h, const double* hu, const doub
   const size_t slots = 2 * (size_t)m->res.nblocks * 16;
   if (m->res.nblocks > 0) { L.add(xbuf); L.add(slots); L.add(4 * (size_t)n); }
   L.add(sizeof(swe::Ctl) * n);
-  if (cudaMalloc((void**)&s->arena.base, L.total) != cudaSuccess) {
-    cudaGetLastError();
+  if (!arena_alloc(s->arena, L.total)) {
     swe_state_destroy(s);
     return SWE_ENOMEM;
   }
-  s->arena.size = L.total;
   if (cuda_failed(cudaMemsetAsync(s->arena.base, 0, L.total, m->stream))) {
     swe_state_destroy(s);
     return SWE_ECUDA;
@@ -1596,7 +1710,7 @@ void swe_state_destroy(swe_state* s) {
   if (s->graph) cudaGraphExecDestroy(s->graph);
   if (s->capture) cudaStreamDestroy(s->capture);
   if (s->host_ctl) cudaFreeHost(s->host_ctl);
-  if (s->arena.base) cudaFree(s->arena.base);
+  arena_free(s->arena);
   delete s;
   if (m) release_mesh(m);
 }

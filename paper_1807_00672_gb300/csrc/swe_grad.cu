@@ -273,7 +273,7 @@ void free_tape(swe_tape* t) {
     if (t->consumed[i]) cudaEventDestroy(t->consumed[i]);
   }
   if (t->side) cudaStreamDestroy(t->side);
-  if (t->arena.base) cudaFree(t->arena.base);
+  arena_free(t->arena);
   swe_mesh* m = t->mesh;
   delete t;
   if (m) release_mesh(m);
@@ -491,12 +491,10 @@ swe_status grad_record(swe_state* s, int64_t n_steps, int64_t checkpoint_every,
   L.add(2 * 8 * (size_t)std::max<int64_t>(1, m->nchunks));
   L.add(sizeof(int));
   L.add(sizeof(unsigned int));
-  if (cudaMalloc((void**)&t->arena.base, L.total) != cudaSuccess) {
-    cudaGetLastError();
+  if (!arena_alloc(t->arena, L.total)) {
     free_tape(t);
     return SWE_ENOMEM;
   }
-  t->arena.size = L.total;
   t->slots.N = t->N;
   t->slots.K = t->K;
   t->slots.nck = t->nck;
