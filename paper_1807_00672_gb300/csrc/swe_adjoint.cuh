@@ -268,6 +268,7 @@ struct AdjArgs {
   const Real* gn2;     // g n^2 per cell
   Real* dgn2;          // accumulated dL/d(g n^2) per cell (read-modify-write)
   Real dt, dt_prev;    // time steps of steps n and n - 1
+  int split;           // parts per tile (Parts; see k_tiled_adjoint)
   int last;            // 1: n = 0
   int* err;            // kErr* bits (timeouts)
   // Gauge seeds of U^n, added to the depth part of mu_out once every block is
@@ -289,7 +290,7 @@ struct AdjLayout {
   uint32_t ext, rec_cap, halo_cap;
   uint32_t off_un, off_tS, off_g0, off_g1, off_g2, off_hidx;
   uint32_t stage;
-  uint32_t off_rho, off_harea, off_slots, off_bars, total;
+  uint32_t off_rho, off_harea, off_list, off_slots, off_bars, total;
 };
 
 inline AdjLayout make_adj_layout(uint32_t w, uint32_t geo_arrays, uint32_t tc, uint32_t ns,
@@ -315,6 +316,7 @@ inline AdjLayout make_adj_layout(uint32_t w, uint32_t geo_arrays, uint32_t tc, u
   o = ns * L.stage;
   L.off_rho = o; o += a16(L.ext * 4 * w);
   L.off_harea = o; o += a16(halo_cap * w);
+  L.off_list = o; o += w == 8 ? a16(rec_cap * 2) : 0u;
   L.off_slots = o; o += a16(3 * (tc + kSlotPad) * 4 * w);
   L.off_bars = o; o += a16(ns * 8);
   L.total = o;
@@ -351,6 +353,13 @@ __global__ void __launch_bounds__(256)
 //       n - 1, whose part of dL/d(g n^2) is accumulated.
 // (A) of the next tile runs right after (C), so two block barriers per tile.
 //
+// Parts (FP64): whole tiles of a small mesh leave SMs idle (40 tiles on 152
+// SMs), so a unit of work is one of `split` parts of a tile: the block stages
+// the whole tile and forms rho of all of it (cheap), lists the records that
+// touch a cell of its part while it does so, and goes through those records
+// and its part's cells only. Faces between two parts are computed twice.
+// adjoint_split chooses.
+//
 // Measured per adjoint step (checkpoints at every step, 64 gauges; before:
 // lambda and U^{n+1} read by every step, friction and velocities redone for
 // halo cells and faces, gauges by one thread): FP32 1.0M cells 54.3 -> 29.2
@@ -364,7 +373,7 @@ __global__ void __launch_bounds__(256)
 template <typename Real, int NT>
 constexpr int adjoint_min_blocks() { return (sizeof(Real) == 4 ? 640 : 256) / NT; }
 
-template <typename Real, int NT, int NS, int CPT>
+template <typename Real, int NT, int NS, int CPT, bool Parts = false>
 __global__ void __launch_bounds__(NT, adjoint_min_blocks<Real, NT>())
     k_tiled_adjoint(DevMesh<Real> m, AdjArgs<Real> A, Num num, AdjLayout L) {
   constexpr int TC = NT * CPT;
@@ -378,7 +387,18 @@ __global__ void __launch_bounds__(NT, adjoint_min_blocks<Real, NT>())
   const Real* __restrict__ area = kRecip ? m.rarea : m.area;
 
   const Chunk ch = m.chunks[blockIdx.x];
-  const int t_first = ch.tile0, n_tiles = ch.ntiles, t_step = ch.stride;
+  // units (tiles, or parts of tiles) ch.tile0 + k ch.stride
+  const int n_tiles = ch.ntiles, split = Parts ? A.split : 1;
+  auto unit = [&](int k) { return ch.tile0 + k * ch.stride; };
+  auto tile_of = [&](int k) { return Parts ? unit(k) / split : unit(k); };
+  // cells [lo, hi) of the tile belong to unit k's part, whole warps of them
+  auto part_of = [&](int k, int& lo, int& hi) {
+    const int p = unit(k) % split;
+    lo = (TC / 32 * p / split) * 32;
+    hi = (TC / 32 * (p + 1) / split) * 32;
+  };
+  uint16_t* list = reinterpret_cast<uint16_t*>(smem + L.off_list);
+  __shared__ int s_list[2];  // records listed for units k, k + 1
   const int cell_end = ch.cell_end;
   const Real dt = A.dt;
   const int tid = threadIdx.x;
@@ -387,6 +407,7 @@ __global__ void __launch_bounds__(NT, adjoint_min_blocks<Real, NT>())
 #pragma unroll
     for (int i = 0; i < NS; ++i) mbar_init(&bar[i], 1);
     fence_mbar_init();
+    s_list[0] = s_list[1] = 0;
   }
   __syncthreads();
 
@@ -463,7 +484,28 @@ __global__ void __launch_bounds__(NT, adjoint_min_blocks<Real, NT>())
   // assignment, so no barrier is needed after its own copies land).
   V4<Real> mu[CPT];
   Real rh[CPT];  // 1 / h of a wet cell, else 0
-  auto phase_a = [&](int st, int tile) {
+  auto phase_a = [&](int st, int k) {
+    const int tile = tile_of(k);
+    if constexpr (Parts) {  // the part's records
+      int lo, hi;
+      part_of(k, lo, hi);
+      const int32_t* codes = reinterpret_cast<const int32_t*>(smem + st * L.stage + L.off_tS);
+      const int nrec = s_nrec[st], lane = tid & 31;
+      auto mine = [&](int code) {  // a cell of the part (padding and walls are no cells)
+        const int j = (-1 - code) & (TC - 1);
+        return code < 0 && code != kSideWall && j >= lo && j < hi;
+      };
+      for (int r0 = tid & ~31; r0 < nrec; r0 += NT) {
+        const int r = r0 + lane;
+        const int packed = r < nrec ? codes[r] : 0;
+        const bool take = r < nrec && (mine(packed >> 16) || mine((int)(int16_t)(packed & 0xffff)));
+        const unsigned m = __ballot_sync(0xffffffffu, take);
+        int at = 0;
+        if (lane == 0 && m) at = atomicAdd(&s_list[k & 1], __popc(m));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (take) list[at + __popc(m & ((1u << lane) - 1u))] = (uint16_t)r;
+      }
+    }
     Real* sun = reinterpret_cast<Real*>(smem + st * L.stage + L.off_un);
     auto to_velocity = [&](Real* c) -> Real {
       const V4<Real> x = ld4(c);
@@ -497,12 +539,12 @@ __global__ void __launch_bounds__(NT, adjoint_min_blocks<Real, NT>())
   if (tid == 0) {
 #pragma unroll
     for (int i = 0; i < NS - 1; ++i)
-      if (i < n_tiles) issue(i, t_first + i * t_step);
+      if (i < n_tiles) issue(i, tile_of(i));
   }
-  if (n_tiles > 0) load_area(t_first);
+  if (n_tiles > 0) load_area(tile_of(0));
   pdl_trigger();
   pdl_wait();
-  if (n_tiles > 0) load_mu(t_first);
+  if (n_tiles > 0) load_mu(tile_of(0));
   if (n_tiles > 0) {
     const bool ok = (tid == 0) ? wait_stage(0) : true;
     if (__syncthreads_or(!ok)) {
@@ -510,7 +552,7 @@ __global__ void __launch_bounds__(NT, adjoint_min_blocks<Real, NT>())
     } else {
       gather_halo(0);
       cp_async_wait_all();
-      phase_a(0, t_first);
+      phase_a(0, 0);
       __syncthreads();
     }
   }
@@ -519,9 +561,9 @@ __global__ void __launch_bounds__(NT, adjoint_min_blocks<Real, NT>())
   // block barriers per tile.
   for (int k = 0; !timeout && k < n_tiles; ++k) {
     const int st = k % NS;
-    const int tile = t_first + k * t_step;
+    const int tile = tile_of(k);
     const bool has_next = k + 1 < n_tiles;
-    if (tid == 0 && k + NS - 1 < n_tiles) issue((k + NS - 1) % NS, tile + (NS - 1) * t_step);
+    if (tid == 0 && k + NS - 1 < n_tiles) issue((k + NS - 1) % NS, tile_of(k + NS - 1));
     const unsigned char* p = smem + st * L.stage;
     const Real* sun = reinterpret_cast<const Real*>(p + L.off_un);
     const int32_t* rS = reinterpret_cast<const int32_t*>(p + L.off_tS);
@@ -540,12 +582,19 @@ __global__ void __launch_bounds__(NT, adjoint_min_blocks<Real, NT>())
       dg[cc] = A.dgn2[base + tid + cc * NT];
     }
     if (has_next) {
-      load_area(tile + t_step);
-      load_mu(tile + t_step);
+      load_area(tile_of(k + 1));
+      load_mu(tile_of(k + 1));
+    }
+    int lo = 0, hi = TC, n_faces = nrec;
+    if constexpr (Parts) {
+      part_of(k, lo, hi);
+      n_faces = s_list[k & 1];
+      if (tid == 0) s_list[(k + 1) & 1] = 0;
     }
 
     // (B) face records
-    for (int r = tid; r < nrec; r += NT) {
+    for (int q = tid; q < n_faces; q += NT) {
+      const int r = Parts ? (int)list[q] : q;
       int32_t packed;
       Real nx, ny, len;
       if constexpr (sizeof(Real) == 4) {
@@ -589,6 +638,7 @@ __global__ void __launch_bounds__(NT, adjoint_min_blocks<Real, NT>())
     for (int cc = 0; cc < CPT; ++cc) {
       const int j = tid + cc * NT;
       if (j >= nc) break;
+      if (Parts && (j < lo || j >= hi)) continue;
       const V4<Real> f0 = ld4(slots + 4 * j);
       const V4<Real> f1 = ld4(slots + 4 * (TC + kSlotPad + j));
       const V4<Real> f2 = ld4(slots + 4 * (2 * (TC + kSlotPad) + j));
@@ -606,7 +656,7 @@ __global__ void __launch_bounds__(NT, adjoint_min_blocks<Real, NT>())
       st4(A.mu_out + 4 * (int64_t)(base + j), lh, lx, ly, lz);
     }
     cp_async_wait_all();
-    if (has_next) phase_a((k + 1) % NS, tile + t_step);
+    if (has_next) phase_a((k + 1) % NS, k + 1);
     __syncthreads();
   }
   if (timeout && tid == 0) {

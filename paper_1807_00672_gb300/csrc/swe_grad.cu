@@ -148,6 +148,12 @@ void launch_adjoint_nt(const swe_mesh* m, const swe::DevMesh<Real>& dm, const sw
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  if constexpr (sizeof(Real) == 8) {
+    if (a.split > 1) {
+      cudaLaunchKernelEx(&cfg, swe::k_tiled_adjoint<Real, NT, 2, CPT, true>, dm, a, num_of(m), L);
+      return;
+    }
+  }
   cudaLaunchKernelEx(&cfg, swe::k_tiled_adjoint<Real, NT, 2, CPT>, dm, a, num_of(m), L);
 }
 
@@ -173,9 +179,9 @@ void launch_adjoint(const swe_mesh* m, const swe::Chunk* chunks, int grid,
 }
 
 // Opts the adjoint kernel into its shared memory; resident blocks per SM.
-template <typename Real, int NT, int CPT>
-int prepare_adjoint_nt(const swe::AdjLayout& L) {
-  auto k = swe::k_tiled_adjoint<Real, NT, 2, CPT>;
+template <typename Real, int NT, int CPT, bool Parts>
+int adjoint_occupancy(const swe::AdjLayout& L) {
+  auto k = swe::k_tiled_adjoint<Real, NT, 2, CPT, Parts>;
   // The limit is a property of the kernel, shared by every mesh that
   // launches it: set it to the device's largest opt-in size (not this
   // layout's), so that a later mesh with a smaller layout cannot lower it
@@ -199,6 +205,13 @@ int prepare_adjoint_nt(const swe::AdjLayout& L) {
   return n;
 }
 
+template <typename Real, int NT, int CPT>
+int prepare_adjoint_nt(const swe::AdjLayout& L) {
+  const int n = adjoint_occupancy<Real, NT, CPT, false>(L);
+  if constexpr (sizeof(Real) == 8) return std::min(n, adjoint_occupancy<Real, NT, CPT, true>(L));
+  return n;
+}
+
 template <typename Real, int CPT>
 int prepare_adjoint_cpt(const swe_mesh* m, const swe::AdjLayout& L) {
   switch (m->tile / CPT) {
@@ -212,6 +225,28 @@ int prepare_adjoint_cpt(const swe_mesh* m, const swe::AdjLayout& L) {
 template <typename Real>
 int prepare_adjoint(const swe_mesh* m, const swe::AdjLayout& L) {
   return m->cpt == 2 ? prepare_adjoint_cpt<Real, 2>(m, L) : prepare_adjoint_cpt<Real, 1>(m, L);
+}
+
+// Parts per tile of the FP64 adjoint (k_tiled_adjoint): the least time on the
+// busiest SM, in units of a tile's 23.5 us. As measured (256-cell tiles), a
+// step costs 0.6 for its launch and latency, and a part its share of the tile
+// and 0.15 for what every part does for the whole tile. us per step, whole
+// tiles and parts: 400 cells (2 tiles, eighths) 32.0 and 20.5, 3,600 (15,
+// eighths) 37.5 and 20.8, 10,000 (40, thirds) 37.6 and 26.5; 22,500 (88) 37.8
+// and 38.3 in thirds, 79,806 (313) 83.2 and 84.0 in halves: whole. FP32 tiles
+// stay whole (10,000 cells: 9.2 us per step, most of it the launch).
+int adjoint_split(int64_t tiles, int sms, int tile_cells) {
+  int best = 1;
+  double least = 0.6 + (double)((tiles + sms - 1) / sms);
+  for (int s = 2; s <= 8 && s <= tile_cells / 32; ++s) {
+    const double part = (double)((tile_cells / 32 + s - 1) / s) * 32 / tile_cells;
+    const double cost = 0.6 + (double)((tiles * s + sms - 1) / sms) * (part + 0.15);
+    if (cost < 0.95 * least) {
+      least = cost;
+      best = s;
+    }
+  }
+  return best;
 }
 
 int grid_for(int64_t n, int cap) {
@@ -245,8 +280,9 @@ struct swe_tape {
   double* gseed_dev = nullptr;
   int32_t* gcells = nullptr;
   swe::GaugeSeeds gauges{};  // gseed_dev by distinct gauge cell
-  swe::Chunk* chunks = nullptr;  // work of the adjoint kernel's blocks
-  int64_t nchunks = 0;
+  swe::Chunk* chunks = nullptr;  // work of the adjoint kernel's blocks, in units of
+  int64_t nchunks = 0;           // 1 / split tiles
+  int split = 1;
   swe::Ctl* ctl = nullptr;      // two replay control words (one per ring)
   double* partial = nullptr;    // two arrays of per-chunk mass partials
   int* err = nullptr;
@@ -398,6 +434,7 @@ swe_status grad_t(swe_tape* t, bool seeds_gauge, int* lam_cur) {
       a.dt = Real(t->dts[j]);
       a.dt_prev = j > 0 ? Real(t->dts[j - 1]) : Real(0);
       a.last = j == 0;
+      a.split = t->split;
       a.err = t->err;
       a.gauges = t->gauges;
       a.gstep = (seeds_gauge && j >= 1) ? (long long)(j - 1) : -1ll;  // lambda^j gets dL/dh^j
@@ -457,12 +494,14 @@ swe_status grad_record(swe_state* s, int64_t n_steps, int64_t checkpoint_every,
   {
     const Scenario& sc = m->scen[0];
     const int64_t resident = (int64_t)m->sms * occ;
-    const int64_t nc = std::min<int64_t>(sc.ntiles, resident);
+    t->split = m->prm.precision == SWE_F64 ? adjoint_split(sc.ntiles, m->sms, m->tile) : 1;
+    const int64_t units = sc.ntiles * t->split;
+    const int64_t nc = std::min<int64_t>(units, resident);
     for (int64_t r = 0; r < nc; ++r) {
       swe::Chunk c{};
       c.scen = 0;
-      c.tile0 = (int32_t)(sc.tile0 + r);
-      c.ntiles = (int32_t)((sc.ntiles - r + nc - 1) / nc);
+      c.tile0 = (int32_t)(sc.tile0 * t->split + r);
+      c.ntiles = (int32_t)((units - r + nc - 1) / nc);
       c.stride = (int32_t)nc;
       c.part = (int32_t)r;
       c.cell_end = (int32_t)(sc.cell0 + sc.ncells);

@@ -384,3 +384,20 @@ def test_recorded_segments_and_a_second_sweep(n_steps, K):
     st.step()  # the state goes on from where the recording ended
     plain.step()
     assert np.array_equal(st.fields()[0], plain.fields()[0])
+
+
+@pytest.mark.parametrize("nx,ny", [(16, 8), (40, 33), (80, 63), (112, 79), (110, 100)])
+def test_adjoint_of_parts_of_tiles(nx, ny):
+    """Meshes of 1, 11, 40, 70 and 86 tiles of 256 cells (the last one partial
+    but for the first mesh), which the FP64 adjoint works in eighths, eighths,
+    thirds, halves and whole: the dot-product test, 1e-10 relative."""
+    c = smooth_wet_case(nx=nx, ny=ny, seed=41)
+    gauges = [1, c.mesh.n_tris - 2]
+    mesh, st, tape = record(c, 4, 2, gauges, tile=256)
+    g = seeds(c, 4, len(gauges), 42)
+    grads = tape.grad(**g)
+    for which in ("h", "hu", "z", "n", "all"):
+        v = directions(c, 43, which)
+        t, gd, _ = oracle_jvp(c, 4, gauges, v)
+        lhs, rhs = pair(g, v, t, gd, grads)
+        assert abs(lhs - rhs) <= 1e-10 * max(abs(lhs), 1e-300), (which, lhs, rhs)
