@@ -341,6 +341,34 @@ int build_host_mesh(const double* xy, int64_t V, const int32_t* tri_in, int64_t 
     area_c[i] = s;
   }
 
+  // The Morton order (of the cells, or for the resident kernel's parts of a
+  // mesh in another order) is sorted on a host thread of its own while the
+  // edges are matched (250,000 cells: 8 of 59 ms).
+  struct ZOrder {
+    std::vector<int32_t> cells;
+    std::thread t;
+    ~ZOrder() {
+      if (t.joinable()) t.join();
+    }
+  } z;
+  auto sort_cells = [&] { return morton_order(xy, V, order == 1 ? tri.data() : tri_in, T); };
+  auto z_order = [&] {
+    if (z.t.joinable()) z.t.join();
+    return (int64_t)z.cells.size() == T ? std::move(z.cells) : sort_cells();
+  };
+  if ((order == 1 || keep_edges) && T >= 20000) {
+    try {
+      z.t = std::thread([&] {
+        try {
+          z.cells = sort_cells();
+        } catch (...) {
+          z.cells.clear();  // sorted (or reported) where it is needed
+        }
+      });
+    } catch (...) {
+    }
+  }
+
   // 2. Half-edges bucketed by their lower node (counting sort), then matched
   //    within each bucket by their upper node.
   std::vector<int64_t> start(V + 1, 0);
@@ -425,7 +453,7 @@ int build_host_mesh(const double* xy, int64_t V, const int32_t* tri_in, int64_t 
   m.perm.resize(T);
   std::iota(m.perm.begin(), m.perm.end(), 0);
   if (order == 1) {
-    m.perm = morton_order(xy, V, tri.data(), T);
+    m.perm = z_order();
   } else if (order == 2) {
     std::vector<int32_t> nbr(3 * T, -1);  // edge neighbours, by face
     for (int64_t i = 0; i < T; ++i)
@@ -437,6 +465,7 @@ int build_host_mesh(const double* xy, int64_t V, const int32_t* tri_in, int64_t 
   } else if (order != 0) {
     return -1;
   }
+  if (keep_edges && order != 1) m.edges.z_order = z_order();
   m.iperm.resize(T);
   for (int64_t j = 0; j < T; ++j) m.iperm[m.perm[j]] = (int32_t)j;
 
@@ -609,7 +638,7 @@ bool build_resident_parts(const HostMesh& m, const double* xy, const int32_t* tr
   // internal cells in Morton order, and the part of each
   std::vector<int32_t> ord, part(T), local(T), nshared(nparts, 0);
   if (!is_morton) {
-    ord = morton_order(xy, m.V, tri, T);
+    ord = (int64_t)ed.z_order.size() == T ? ed.z_order : morton_order(xy, m.V, tri, T);
     for (int64_t r = 0; r < T; ++r) ord[r] = m.iperm[ord[r]];
   }
   auto cell_at = [&](int64_t r) { return is_morton ? (int32_t)r : ord[r]; };

@@ -30,9 +30,10 @@ int guarded(F&& body) noexcept {
 constexpr int32_t kWall = INT32_MIN;
 
 // Edges by caller cell (kept in HostMesh on request): left (lower) and right
-// cell, outward normal and length, and each half-edge's edge.
+// cell, outward normal and length, and each half-edge's edge; for meshes not
+// in Morton order that order of the caller cells.
 struct HostEdges {
-  std::vector<int32_t> cL, cR, of_half;
+  std::vector<int32_t> cL, cR, of_half, z_order;
   std::vector<double> nx, ny, len;
 };
 
