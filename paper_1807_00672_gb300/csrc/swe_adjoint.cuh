@@ -34,27 +34,13 @@
 
 namespace swe {
 
-// dt h^{-7/3} and 1 / h of a wet depth.
-__device__ __forceinline__ void depth_powers(float h, float dt, float& ch, float& rh) {
-  ch = Ops<float>::friction(dt, 1.0f, 1.0f, h);
-  rh = rcp_approx(h);
-}
-__device__ __forceinline__ void depth_powers(double h, double dt, double& ch, double& rh) {
-  const double y = icbrt_nr(h), y2 = mul_rn(y, y);
-  rh = mul_rn(y2, y);
-  ch = mul_rn(dt, mul_rn(mul_rn(y2, y2), rh));
-}
-
-// Signs by value; FP64 from the bit patterns (a comparison costs as much of
-// the FP64 pipe as a multiply-add).
-__device__ __forceinline__ bool below0(float x) { return x < 0.0f; }
+// Signs and orders of doubles from their bit patterns (a comparison costs as
+// much of the FP64 pipe as a multiply-add).
 __device__ __forceinline__ bool below0(double x) {
   return (unsigned long long)__double_as_longlong(x) > 0x8000000000000000ull;
 }
-__device__ __forceinline__ bool above0(float x) { return x > 0.0f; }
 __device__ __forceinline__ bool above0(double x) { return __double_as_longlong(x) > 0; }
 // a >= b
-__device__ __forceinline__ bool at_least(float a, float b) { return a >= b; }
 __device__ __forceinline__ bool at_least(double a, double b) {
   const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b);
   const long long ka = ia ^ ((ia >> 63) & 0x7fffffffffffffffll);
@@ -62,20 +48,44 @@ __device__ __forceinline__ bool at_least(double a, double b) {
   return ka >= kb || ((ia | ib) << 1) == 0;  // -0 and +0 are equal
 }
 // 2 x for a normal x > 0 (or 0 with pos false)
-__device__ __forceinline__ float twice(float x, bool) { return x + x; }
 __device__ __forceinline__ double twice(double x, bool pos) {
   return pos ? __hiloint2double(__double2hiint(x) + 0x00100000, __double2loint(x)) : 0.0;
 }
 
 // dL/dU* of one cell from its post-step state (h1, q1x, q1y) and lambda:
-// mu (3 values) and the derivative with respect to its g n^2 (left 0 where
-// g n^2 is 0: it only enters dL/dn, multiplied by n).
-template <typename Real>
-__device__ __forceinline__ void cell_vjp(Real h1, Real q1x, Real q1y, Real lh, Real lx, Real ly,
-                                         Real gn2, Real dt, const Num& num, Real& mh, Real& mx,
-                                         Real& my, Real& bgn2) {
-  using O = Ops<Real>;
-  const Real zero = Real(0);
+// mu (3 values) and the derivative with respect to its g n^2.
+__device__ __forceinline__ void cell_vjp(float h1, float q1x, float q1y, float lh, float lx, float ly,
+                                         float gn2, float dt, const Num& num, float& mh, float& mx,
+                                         float& my, float& bgn2) {
+  using O = Ops<float>;
+  const float zero = 0.0f;
+  if (O::wet(h1, num)) {
+    const float q1n = O::sqrt_(q1x * q1x + q1y * q1y);
+    const float ch = O::friction(dt, 1.0f, 1.0f, h1);  // dt h^{-7/3}
+    const float c = ch * gn2;
+    const float cq = c * q1n;        // (d - 1) / d
+    const float rd = 1.0f - cq;   // 1 / d
+    const float ql = q1x * lx + q1y * ly;
+    const float k = q1n > zero ? O::div(c * ql, q1n) : zero;
+    mx = rd * (lx - k * q1x);
+    my = rd * (ly - k * q1y);
+    mh = lh + float(7.0 / 3.0) * O::div(cq, h1) * ql;
+    bgn2 = -q1n * ch * ql;
+  } else {
+    mh = lh;
+    mx = zero;
+    my = zero;
+    bgn2 = zero;
+  }
+}
+
+// FP64: fewer FP64 instructions; the last output is left 0 where g n^2 is 0
+// (it only enters dL/dn, multiplied by n).
+__device__ __forceinline__ void cell_vjp(double h1, double q1x, double q1y, double lh, double lx,
+                                         double ly, double gn2, double dt, const Num& num, double& mh,
+                                         double& mx, double& my, double& bgn2) {
+  using O = Ops<double>;
+  const double zero = 0.0;
   mh = lh;
   mx = zero;
   my = zero;
@@ -84,26 +94,28 @@ __device__ __forceinline__ void cell_vjp(Real h1, Real q1x, Real q1y, Real lh, R
   mx = lx;
   my = ly;
   if (!above0(gn2)) return;
-  const Real q1n = O::sqrt_(fma_rn(q1x, q1x, q1y * q1y));
-  Real ch, rh;
-  depth_powers(h1, dt, ch, rh);
-  const Real c = ch * gn2;
-  const Real cq = c * q1n;        // (d - 1) / d
-  const Real rd = Real(1) - cq;   // 1 / d
-  const Real ql = fma_rn(q1x, lx, q1y * ly);
-  const Real k = above0(q1n) ? O::div(c * ql, q1n) : zero;
+  const double q1n = O::sqrt_(fma_rn(q1x, q1x, q1y * q1y));
+  const double y = icbrt_nr(h1), y2 = mul_rn(y, y);  // h^{-1/3}
+  const double rh = mul_rn(y2, y);                   // 1 / h
+  const double ch = mul_rn(dt, mul_rn(mul_rn(y2, y2), rh));
+  const double c = ch * gn2;
+  const double cq = c * q1n;        // (d - 1) / d
+  const double rd = 1.0 - cq;   // 1 / d
+  const double ql = fma_rn(q1x, lx, q1y * ly);
+  const double k = above0(q1n) ? O::div(c * ql, q1n) : zero;
   mx = rd * fma_rn(-k, q1x, lx);
   my = rd * fma_rn(-k, q1y, ly);
-  mh = fma_rn(Real(7.0 / 3.0) * (cq * rh), ql, lh);
+  mh = fma_rn((7.0 / 3.0) * (cq * rh), ql, lh);
   bgn2 = -(q1n * ch) * ql;
 }
 
 // Vector-Jacobian product of one face, with both sides' contributions:
-// inputs the sides' cells (h, u, v, z) as the forward step reads them
-// (velocities formed once per cell, 0 on a dry one), the geometry, and rho =
-// dL/dR of side A (the face adds c_A to R_A) and side B (the face subtracts
-// c_B from R_B); outputs gA, gB = dL/d(h, u, v, z) of each side through this
-// face. The face is the clamped form of the flux the tiled steps compute
+// inputs the sides' cells as staged, the geometry, and rho = dL/dR of side A
+// (the face adds c_A to R_A) and side B (the face subtracts c_B from R_B);
+// outputs gA, gB through this face. FP32: cells (h, hu, hv, z), outputs
+// dL/d(h, hu, hv, z). FP64: cells (h, u, v, z), velocities formed once per
+// cell (0 on a dry one), outputs dL/d(h, u, v, z), taken back to hu, hv once
+// per cell. The face is the clamped form of the flux the tiled steps compute
 // (face_flux_f32, face_flux_f64): one HLL formula with the clamped speeds
 // S- = min(S_A, 0), S+ = max(S_B, 0), the dry side's normal velocity replaced
 // by un_B - 2 c_B (or un_A + 2 c_A) in the wave-speed estimates, the
@@ -116,6 +128,135 @@ __device__ __forceinline__ void cell_vjp(Real h1, Real q1x, Real q1y, Real lh, R
 // as S_A >= 0 and S_B = 0 as S_B <= 0. For a wall B is ignored (the mirror of
 // A folds into gA, gB = 0).
 //
+// FP32 differentiates the formulas as they stand: the shorter FP64 form below
+// was no faster in FP32 (29.2 and 29.3 us per step of 1.0M cells), whose bound
+// is not its arithmetic.
+template <bool Wall>
+__device__ __forceinline__ void face_vjp(const V4<float>& A, const V4<float>& B, float nx, float ny,
+                                         float len, const Num& num, float rA0, float rA1, float rA2,
+                                         float rB0, float rB1, float rB2, float gA[4], float gB[4]) {
+  using O = Ops<float>;
+  const float zero = 0.0f, half = 0.5f, quarter = 0.25f;
+  const float g = float(num.g), hg = half * g;
+  // ---- forward, keeping what the reverse sweep needs
+  const float rA = O::wet(A.x, num) ? O::div(1.0f, A.x) : zero;  // 0 on a dry cell
+  const float uA = A.y * rA, vA = A.z * rA;
+  const float unA = uA * nx + vA * ny;
+  const float utA = vA * nx - uA * ny;
+  float hB, zB, unB, utB, uB = zero, vB = zero, rB = zero;
+  if (Wall) {
+    hB = A.x; zB = A.w; unB = -unA; utB = utA;
+  } else {
+    rB = O::wet(B.x, num) ? O::div(1.0f, B.x) : zero;
+    uB = B.y * rB;
+    vB = B.z * rB;
+    hB = B.x; zB = B.w;
+    unB = uB * nx + vB * ny;
+    utB = vB * nx - uB * ny;
+  }
+  const bool zsA = A.w >= zB;  // max(zA, zB) taken from A on a tie
+  const float zs = zsA ? A.w : zB;
+  const float xA = A.x + A.w - zs, xB = hB + zB - zs;
+  const bool wetA = O::wet(xA, num), wetB = O::wet(xB, num);  // reconstructed sides wet
+  const float hAs = wetA ? xA : zero, hBs = wetB ? xB : zero;
+  const float cA = O::sqrt_(g * hAs), cB = O::sqrt_(g * hBs);
+  const float vnA = wetA ? unA : unB - 2.0f * cB;
+  const float vnB = wetB ? unB : unA + 2.0f * cA;
+  const float us = (vnA + vnB) * half + cA - cB;
+  const float cs = (cA + cB) * half + (vnA - vnB) * quarter;
+  const float a1 = vnA - cA, a2 = us - cs, b1 = vnB + cB, b2 = us + cs;
+  const bool firstA = a1 <= a2, firstB = b1 >= b2;
+  const float SA = firstA ? a1 : a2, SB = firstB ? b1 : b2;
+  const bool negA = SA < zero, posB = SB > zero;
+  const float Sm = negA ? SA : zero, Sp = posB ? SB : zero;
+  const float qA = hAs * unA, qB = hBs * unB;
+  const float FA1 = qA * unA + hg * hAs * hAs, FB1 = qB * unB + hg * hBs * hBs;
+  const bool live = wetA || wetB;  // both sides dry: F = 0 whatever the speeds
+  const float inv = live ? O::div(1.0f, Sp - Sm) : zero;
+  const float SS = Sm * Sp, dh = hBs - hAs, dq = qB - qA;
+  const float N0 = Sp * qA - Sm * qB + SS * dh;
+  const float N1 = Sp * FA1 - Sm * FB1 + SS * dq;
+  const float F0 = N0 * inv;
+  const bool upA = F0 >= zero;  // transverse momentum from A where F0 >= 0
+
+  // ---- reverse sweep
+  // residual contributions: A gets +l (F0, Fx + PA nx, Fy + PA ny), B gets
+  // -l (F0, Fx + PB nx, Fy + PB ny), Fx = F1 nx - F2 ny, Fy = F1 ny + F2 nx
+  const float bFx = len * (rA1 - rB1), bFy = len * (rA2 - rB2);
+  const float bF1 = bFx * nx + bFy * ny;
+  float bF0 = zero, bF2 = zero;
+  if (!Wall) {
+    bF0 = len * (rA0 - rB0);
+    bF2 = bFy * nx - bFx * ny;
+  }
+  const float bPA = len * (rA1 * nx + rA2 * ny);
+  const float bPB = Wall ? zero : -len * (rB1 * nx + rB2 * ny);
+  // P = g/2 (h^2 - h*^2)
+  float bhA = g * A.x * bPA, bhB = g * hB * bPB;
+  float bhAs = -g * hAs * bPA, bhBs = -g * hBs * bPB;
+  // F2 = F0 ut
+  bF0 += bF2 * (upA ? utA : utB);
+  const float but = bF2 * F0;
+  float butA = upA ? but : zero, butB = upA ? zero : but;
+  // F0 = N0 / D, F1 = N1 / D, D = S+ - S-
+  const float bN0 = bF0 * inv, bN1 = bF1 * inv;
+  const float bD = -(bF0 * N0 + bF1 * N1) * inv * inv;
+  const float bSp = bD + bN0 * (qA + Sm * dh) + bN1 * (FA1 + Sm * dq);
+  const float bSm = -bD + bN0 * (Sp * dh - qB) + bN1 * (Sp * dq - FB1);
+  float bqA = bN0 * Sp - bN1 * SS, bqB = bN1 * SS - bN0 * Sm;
+  bhBs += bN0 * SS;
+  bhAs -= bN0 * SS;
+  const float bFA1 = bN1 * Sp, bFB1 = -bN1 * Sm;
+  // F1 of each side = q un + g/2 h*^2, q = h* un
+  bqA += bFA1 * unA;
+  bqB += bFB1 * unB;
+  float bunA = bFA1 * qA + bqA * hAs, bunB = bFB1 * qB + bqB * hBs;
+  bhAs += bFA1 * g * hAs + bqA * unA;
+  bhBs += bFB1 * g * hBs + bqB * unB;
+  // S- = min(S_A, 0), S+ = max(S_B, 0); the speed estimates
+  const float bSA = negA ? bSm : zero, bSB = posB ? bSp : zero;
+  float bvnA = zero, bvnB = zero, bcA = zero, bcB = zero, bus = zero, bcs = zero;
+  if (firstA) { bvnA += bSA; bcA -= bSA; } else { bus += bSA; bcs -= bSA; }
+  if (firstB) { bvnB += bSB; bcB += bSB; } else { bus += bSB; bcs += bSB; }
+  bvnA += half * bus + quarter * bcs;
+  bvnB += half * bus - quarter * bcs;
+  bcA += bus + half * bcs;
+  bcB += half * bcs - bus;
+  // a dry side's velocity in the estimates
+  if (wetA) { bunA += bvnA; } else { bunB += bvnA; bcB -= 2.0f * bvnA; }
+  if (wetB) { bunB += bvnB; } else { bunA += bvnB; bcA += 2.0f * bvnB; }
+  // c = sqrt(g h*): dc/dh* = g / (2 c) on a wet side (c = 0 and no term on a dry one)
+  if (wetA) bhAs += bcA * O::div(hg, cA);
+  if (wetB) bhBs += bcB * O::div(hg, cB);
+  // reconstruction h* = h + z - max(zA, zB) where it stays wet
+  float bzA = zero, bzB = zero, bzs = zero;
+  if (wetA) { bhA += bhAs; bzA += bhAs; bzs -= bhAs; }
+  if (wetB) { bhB += bhBs; bzB += bhBs; bzs -= bhBs; }
+  if (zsA) bzA += bzs; else bzB += bzs;
+  if (Wall) {  // B mirrors A: hB = hA, zB = zA, unB = -unA, utB = utA
+    bhA += bhB;
+    bzA += bzB;
+    bunA -= bunB;
+    butA += butB;
+  }
+  // face frame -> x, y velocities -> conserved variables (u = hu r, r = 1/h
+  // on a wet cell, 0 on a dry one)
+  const float buA = bunA * nx - butA * ny, bvA = bunA * ny + butA * nx;
+  gA[0] = bhA - (buA * uA + bvA * vA) * rA;
+  gA[1] = buA * rA;
+  gA[2] = bvA * rA;
+  gA[3] = bzA;
+  if (Wall) {
+    gB[0] = zero; gB[1] = zero; gB[2] = zero; gB[3] = zero;
+  } else {
+    const float buB = bunB * nx - butB * ny, bvB = bunB * ny + butB * nx;
+    gB[0] = bhB - (buB * uB + bvB * vB) * rB;
+    gB[1] = buB * rB;
+    gB[2] = bvB * rB;
+    gB[3] = bzB;
+  }
+}
+
 // FP64: the FP64 pipe bounds the adjoint as it bounds the step, so the sweep
 // is arranged for few FP64 instructions (115 of them; about 175 when each
 // face formed its velocities and differentiated N / D):
@@ -127,79 +268,79 @@ __device__ __forceinline__ void cell_vjp(Real h1, Real q1x, Real q1y, Real lh, R
 //   - z enters through the higher side only: one side's part, negated for
 //     the other;
 //   - signs and orders from bit patterns.
-template <typename Real, bool Wall>
-__device__ __forceinline__ void face_vjp(const V4<Real>& A, const V4<Real>& B, Real nx, Real ny,
-                                         Real len, const Num& num, Real rA0, Real rA1, Real rA2,
-                                         Real rB0, Real rB1, Real rB2, Real gA[4], Real gB[4]) {
-  using O = Ops<Real>;
-  const Real zero = Real(0), k34 = Real(0.75), two = Real(2);
-  const Real g = Real(num.g), hg = Real(0.5) * g;
+template <bool Wall>
+__device__ __forceinline__ void face_vjp(const V4<double>& A, const V4<double>& B, double nx, double ny,
+                                         double len, const Num& num, double rA0, double rA1, double rA2,
+                                         double rB0, double rB1, double rB2, double gA[4], double gB[4]) {
+  using O = Ops<double>;
+  const double zero = 0.0, k34 = 0.75, two = 2.0;
+  const double g = num.g, hg = 0.5 * g;
   // ---- forward
-  const Real unA = fma_rn(A.y, nx, A.z * ny);
-  const Real hB = Wall ? A.x : B.x, zB = Wall ? A.w : B.w;
-  const Real unB = Wall ? -unA : fma_rn(B.y, nx, B.z * ny);
+  const double unA = fma_rn(A.y, nx, A.z * ny);
+  const double hB = Wall ? A.x : B.x, zB = Wall ? A.w : B.w;
+  const double unB = Wall ? -unA : fma_rn(B.y, nx, B.z * ny);
   const bool zsA = Wall || at_least(A.w, zB);  // max(zA, zB) taken from A on a tie
-  const Real zs = zsA ? A.w : zB;
-  const Real xA = sub_rn(add_rn(A.x, A.w), zs), xB = Wall ? xA : sub_rn(add_rn(hB, zB), zs);
+  const double zs = zsA ? A.w : zB;
+  const double xA = sub_rn(add_rn(A.x, A.w), zs), xB = Wall ? xA : sub_rn(add_rn(hB, zB), zs);
   const bool wetA = O::wet(xA, num), wetB = O::wet(xB, num);  // reconstructed sides wet
-  const Real hAs = wetA ? xA : zero, hBs = wetB ? xB : zero;
-  const Real pA = hg * hAs, pB = Wall ? pA : hg * hBs;
-  const Real cA = O::sqrt_(twice(pA, wetA)), cB = Wall ? cA : O::sqrt_(twice(pB, wetB));
-  Real vnA = unA, vnB = unB;
+  const double hAs = wetA ? xA : zero, hBs = wetB ? xB : zero;
+  const double pA = hg * hAs, pB = Wall ? pA : hg * hBs;
+  const double cA = O::sqrt_(twice(pA, wetA)), cB = Wall ? cA : O::sqrt_(twice(pB, wetB));
+  double vnA = unA, vnB = unB;
   if (!(wetA && wetB)) {
     if (!wetA) vnA = fma_rn(-two, cB, unB);
     if (!wetB) vnB = fma_rn(two, cA, unA);
   }
-  const Real dv = vnB - vnA, dc = cA - cB;
-  const Real eA = fma_rn(two, dc, dv), eB = fma_rn(two, dc, -dv);
+  const double dv = vnB - vnA, dc = cA - cB;
+  const double eA = fma_rn(two, dc, dv), eB = fma_rn(two, dc, -dv);
   const bool secA = below0(eA), secB = above0(eB);  // the star-region estimate is the extreme one
-  const Real SA = fma_rn(k34, secA ? eA : zero, vnA - cA);
-  const Real SB = fma_rn(k34, secB ? eB : zero, vnB + cB);
+  const double SA = fma_rn(k34, secA ? eA : zero, vnA - cA);
+  const double SB = fma_rn(k34, secB ? eB : zero, vnB + cB);
   const bool negA = below0(SA), posB = above0(SB);
-  const Real Sm = negA ? SA : zero, Sp = posB ? SB : zero;
-  const Real qA = hAs * unA, qB = hBs * unB;
-  const Real dh = hBs - hAs, dq = qB - qA;
-  const Real dF = Wall ? zero : fma_rn(qB, unB, pB * hBs) - fma_rn(qA, unA, pA * hAs);
+  const double Sm = negA ? SA : zero, Sp = posB ? SB : zero;
+  const double qA = hAs * unA, qB = hBs * unB;
+  const double dh = hBs - hAs, dq = qB - qA;
+  const double dF = Wall ? zero : fma_rn(qB, unB, pB * hBs) - fma_rn(qA, unA, pA * hAs);
   const bool live = wetA || wetB;  // both sides dry: F = 0 whatever the speeds
-  const Real inv = live ? O::rcp(Sp - Sm) : zero;
-  const Real wm = Sm * inv, wp = Sp * inv, ws = Sm * wp;
+  const double inv = live ? O::rcp(Sp - Sm) : zero;
+  const double wm = Sm * inv, wp = Sp * inv, ws = Sm * wp;
 
   // ---- reverse sweep
   // residual contributions: A gets +l (F0, Fx + PA nx, Fy + PA ny), B gets
   // -l (F0, Fx + PB nx, Fy + PB ny), Fx = F1 nx - F2 ny, Fy = F1 ny + F2 nx
-  const Real gx = len * nx, gy = len * ny;
-  const Real d1 = Wall ? rA1 : rA1 - rB1, d2 = Wall ? rA2 : rA2 - rB2;
-  const Real bF1 = fma_rn(d1, gx, d2 * gy);
+  const double gx = len * nx, gy = len * ny;
+  const double d1 = Wall ? rA1 : rA1 - rB1, d2 = Wall ? rA2 : rA2 - rB2;
+  const double bF1 = fma_rn(d1, gx, d2 * gy);
   // P = g/2 (h^2 - h*^2)
-  const Real gPA = g * (Wall ? bF1 : fma_rn(rA1, gx, rA2 * gy));
-  const Real gPB = Wall ? zero : -g * fma_rn(rB1, gx, rB2 * gy);
-  Real bF0 = zero, but = zero;
+  const double gPA = g * (Wall ? bF1 : fma_rn(rA1, gx, rA2 * gy));
+  const double gPB = Wall ? zero : -g * fma_rn(rB1, gx, rB2 * gy);
+  double bF0 = zero, but = zero;
   bool upA = true;
   if (!Wall) {
     // F2 = F0 ut, ut of the upwind side
-    const Real F0 = fma_rn(ws, dh, fma_rn(wp, qA, -(wm * qB)));
+    const double F0 = fma_rn(ws, dh, fma_rn(wp, qA, -(wm * qB)));
     upA = !below0(F0);
-    const Real uu = upA ? A.y : B.y, vv = upA ? A.z : B.z;
-    const Real bF2 = fma_rn(d2, gx, -(d1 * gy));
+    const double uu = upA ? A.y : B.y, vv = upA ? A.z : B.z;
+    const double bF2 = fma_rn(d2, gx, -(d1 * gy));
     bF0 = fma_rn(bF2, fma_rn(vv, nx, -(uu * ny)), len * (rA0 - rB0));
     but = bF2 * F0;
   }
   // F0 (states q, h) and F1 (states F, q) of the two sides and the speeds
-  const Real P = Wall ? zero : fma_rn(bF1, dF, bF0 * dq) * inv;
-  const Real Q = (Wall ? bF1 * dq : fma_rn(bF1, dq, bF0 * dh)) * inv;
-  const Real bSB = posB ? wm * fma_rn(-Sm, Q, P) : zero;
-  const Real bSA = negA ? wp * fma_rn(Sp, Q, -P) : zero;
-  const Real bFA = bF1 * wp, bFB = -(bF1 * wm), s1 = bF1 * ws, s0 = Wall ? zero : bF0 * ws;
-  const Real bqA = fma_rn(bFA, unA, Wall ? -s1 : fma_rn(bF0, wp, -s1));
-  const Real bqB = fma_rn(bFB, unB, Wall ? s1 : fma_rn(-bF0, wm, s1));
-  Real bunA = fma_rn(bqA, hAs, bFA * qA), bunB = fma_rn(bqB, hBs, bFB * qB);
-  Real bhAs = fma_rn(fma_rn(g, bFA, -gPA), hAs, fma_rn(bqA, unA, -s0));
-  Real bhBs = fma_rn(Wall ? g * bFB : fma_rn(g, bFB, -gPB), hBs, fma_rn(bqB, unB, s0));
+  const double P = Wall ? zero : fma_rn(bF1, dF, bF0 * dq) * inv;
+  const double Q = (Wall ? bF1 * dq : fma_rn(bF1, dq, bF0 * dh)) * inv;
+  const double bSB = posB ? wm * fma_rn(-Sm, Q, P) : zero;
+  const double bSA = negA ? wp * fma_rn(Sp, Q, -P) : zero;
+  const double bFA = bF1 * wp, bFB = -(bF1 * wm), s1 = bF1 * ws, s0 = Wall ? zero : bF0 * ws;
+  const double bqA = fma_rn(bFA, unA, Wall ? -s1 : fma_rn(bF0, wp, -s1));
+  const double bqB = fma_rn(bFB, unB, Wall ? s1 : fma_rn(-bF0, wm, s1));
+  double bunA = fma_rn(bqA, hAs, bFA * qA), bunB = fma_rn(bqB, hBs, bFB * qB);
+  double bhAs = fma_rn(fma_rn(g, bFA, -gPA), hAs, fma_rn(bqA, unA, -s0));
+  double bhBs = fma_rn(Wall ? g * bFB : fma_rn(g, bFB, -gPB), hBs, fma_rn(bqB, unB, s0));
   // the speed estimates
-  const Real tA = secA ? k34 * bSA : zero, tB = secB ? k34 * bSB : zero;
-  const Real td = tA - tB, ts = tA + tB;
-  const Real bvA = bSA - td, bvB = bSB + td;
-  Real bcA = fma_rn(two, ts, -bSA), bcB = fma_rn(-two, ts, bSB);
+  const double tA = secA ? k34 * bSA : zero, tB = secB ? k34 * bSB : zero;
+  const double td = tA - tB, ts = tA + tB;
+  const double bvA = bSA - td, bvB = bSB + td;
+  double bcA = fma_rn(two, ts, -bSA), bcB = fma_rn(-two, ts, bSB);
   if (wetA && wetB) {
     bunA += bvA;
     bunB += bvB;
@@ -211,13 +352,13 @@ __device__ __forceinline__ void face_vjp(const V4<Real>& A, const V4<Real>& B, R
   bhAs = wetA ? fma_rn(bcA * hg, O::rcp(cA), bhAs) : zero;
   bhBs = wetB ? fma_rn(bcB * hg, Wall ? O::rcp(cA) : O::rcp(cB), bhBs) : zero;
   // reconstruction h* = h + z - max(zA, zB) where it stays wet
-  Real bhA = fma_rn(A.x, gPA, bhAs);
+  double bhA = fma_rn(A.x, gPA, bhAs);
   if (Wall) {  // B mirrors A: hB = hA, zB = zA, unB = -unA, utB = utA
     bhA += bhBs;
     bunA -= bunB;
   }
   // face frame -> x, y
-  const Real tx = but * ny, ty = but * nx;
+  const double tx = but * ny, ty = but * nx;
   gA[0] = bhA;
   gA[1] = Wall ? bunA * nx : fma_rn(bunA, nx, upA ? -tx : zero);
   gA[2] = Wall ? bunA * ny : fma_rn(bunA, ny, upA ? ty : zero);
@@ -232,30 +373,24 @@ __device__ __forceinline__ void face_vjp(const V4<Real>& A, const V4<Real>& B, R
   }
 }
 
-// Loss seeds of the gauges: the ncells distinct cells that hold gauges, and
-// for each the gauges in it (index[first[c]] .. index[first[c + 1] - 1], in
+// Loss seeds of the gauges: the ncells distinct cells that hold gauges,
+// ascending, those of tile t at tile_first[t] .. tile_first[t + 1] - 1, and for
+// each the gauges in it (index[first[c]] .. index[first[c + 1] - 1], in
 // ascending order); seed[k G + j] is dL/d(depth at gauge j after step k).
 struct GaugeSeeds {
   const int32_t* cells;
   const int32_t* first;
   const int32_t* index;
+  const int32_t* tile_first;
   const double* seed;
   int G, ncells;
 };
 
-// Adds the seeds of step k to the depth adjoint of interleaved cells: one
-// thread per distinct cell, so that repeated gauge cells add up in a fixed
-// order. (One thread for all of them: 64 gauges added 16 us to an adjoint
-// step of 1M triangles, 54 us, each a dependent trip to L2.)
+// The seeds of step k of distinct gauge cell c, added to v in a fixed order.
 template <typename Real>
-__device__ __forceinline__ void add_gauge_seeds(Real* lam, const GaugeSeeds& g, long long k, int tid,
-                                                int nthreads) {
-  for (int c = tid; c < g.ncells; c += nthreads) {
-    Real* p = lam + 4 * (int64_t)g.cells[c];
-    Real v = __ldcg(p);  // other blocks wrote it
-    for (int q = g.first[c]; q < g.first[c + 1]; ++q) v += Real(g.seed[k * g.G + g.index[q]]);
-    *p = v;
-  }
+__device__ __forceinline__ Real add_seeds(Real v, const GaugeSeeds& g, long long k, int c) {
+  for (int q = g.first[c]; q < g.first[c + 1]; ++q) v += Real(g.seed[k * g.G + g.index[q]]);
+  return v;
 }
 
 // Inputs and outputs of one adjoint launch, step n (interleaved cells,
@@ -271,13 +406,12 @@ struct AdjArgs {
   int split;           // parts per tile (Parts; see k_tiled_adjoint)
   int last;            // 1: n = 0
   int* err;            // kErr* bits (timeouts)
-  // Gauge seeds of U^n, added to the depth part of mu_out once every block is
-  // done (by the last block); gstep < 0 adds nothing. (The transposed
-  // friction adds its part to the depth derivative, so the seed may come
-  // after it.) ticket: a zeroed counter.
+  // Gauge seeds of U^n, added to dL/dh of their cells before the transposed
+  // friction of step n - 1 (by the cell's own thread: one thread for all of
+  // them at the end of the launch cost 16 us per step with 64 gauges, a
+  // dependent trip to L2 each); gstep < 0 adds nothing.
   GaugeSeeds gauges;
   long long gstep;
-  unsigned int* ticket;
 };
 
 // Shared-memory plan of k_tiled_adjoint. Per stage: the tile's and its
@@ -333,7 +467,7 @@ __global__ void __launch_bounds__(256)
        i += (int64_t)gridDim.x * blockDim.x) {
     const V4<Real> c = ld4(u1 + 4 * i), l = ld4(lam + 4 * i);
     Real mh, mx, my, b;
-    cell_vjp<Real>(c.x, c.y, c.z, l.x, l.y, l.z, gn2[i], dt, num, mh, mx, my, b);
+    cell_vjp(c.x, c.y, c.z, l.x, l.y, l.z, gn2[i], dt, num, mh, mx, my, b);
     st4(lam + 4 * i, mh, mx, my, l.w);
     dgn2[i] = b;
   }
@@ -361,12 +495,12 @@ __global__ void __launch_bounds__(256)
 // adjoint_split chooses.
 //
 // Measured per adjoint step (checkpoints at every step, 64 gauges; before:
-// lambda and U^{n+1} read by every step, friction and velocities redone for
-// halo cells and faces, gauges by one thread): FP32 1.0M cells 54.3 -> 29.2
-// us, 160,000 cells 28.0 -> 12.0, 10,000 cells 12.2 -> 9.6; FP64 (16 gauges)
-// 79,806 cells 153 -> 83, 10,000 cells 58 -> 38. FP64 is bound by the FP64
-// pipe, and by tiles not dividing over the SMs on small meshes; FP32 by
-// instruction issue and the two barriers per tile.
+// lambda and U^{n+1} read by every step, friction redone for halo cells,
+// FP64 velocities per face, gauges by one thread at the end): FP32 1.0M cells
+// 54.3 -> 29.3 us, 160,000 cells 28.0 -> 11.3, 10,000 cells 12.2 -> 8.7; FP64
+// (16 gauges) 79,806 cells 153 -> 82, 10,000 cells 58 -> 25. FP64 is bound by
+// the FP64 pipe, and by tiles not dividing over the SMs on small meshes; FP32
+// by instruction issue and the two barriers per tile.
 //
 // Registers are capped so that 640 FP32 threads (5 blocks of 128 with
 // 256-cell tiles, which their shared memory also allows) share an SM.
@@ -377,14 +511,14 @@ template <typename Real, int NT, int NS, int CPT, bool Parts = false>
 __global__ void __launch_bounds__(NT, adjoint_min_blocks<Real, NT>())
     k_tiled_adjoint(DevMesh<Real> m, AdjArgs<Real> A, Num num, AdjLayout L) {
   constexpr int TC = NT * CPT;
-  constexpr bool kRecip = sizeof(Real) == 8;  // FP64 meshes keep 1 / area
+  constexpr bool kF64 = sizeof(Real) == 8;  // velocities per cell, 1 / area from the mesh
   __shared__ int s_nrec[NS], s_nh[NS];
   extern __shared__ __align__(128) unsigned char smem[];
   Real* rho = reinterpret_cast<Real*>(smem + L.off_rho);      // [ext][4]
   Real* harea = reinterpret_cast<Real*>(smem + L.off_harea);  // [halo_cap]
   Real* slots = reinterpret_cast<Real*>(smem + L.off_slots);  // [3 (TC + kSlotPad)][4]
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L.off_bars);
-  const Real* __restrict__ area = kRecip ? m.rarea : m.area;
+  const Real* __restrict__ area = kF64 ? m.rarea : m.area;
 
   const Chunk ch = m.chunks[blockIdx.x];
   // units (tiles, or parts of tiles) ch.tile0 + k ch.stride
@@ -478,7 +612,7 @@ __global__ void __launch_bounds__(NT, adjoint_min_blocks<Real, NT>())
 #pragma unroll
     for (int cc = 0; cc < CPT; ++cc) nmu[cc] = ld4(A.mu_in + 4 * (b0 + tid + cc * NT));
   };
-  auto scale = [&](Real a) { return kRecip ? -(dt * a) : -Ops<Real>::div(dt, a); };
+  auto scale = [&](Real a) { return kF64 ? -(dt * a) : -Ops<Real>::div(dt, a); };
   // (A) of a tile: the thread's own cells from the registers load_area and
   // load_mu filled, and the halo cells this thread gathered (gather_halo's
   // assignment, so no barrier is needed after its own copies land).
@@ -520,7 +654,7 @@ __global__ void __launch_bounds__(NT, adjoint_min_blocks<Real, NT>())
       mu[cc] = nmu[cc];
       const Real a = j < nc ? scale(nar[cc]) : Real(0);  // padding: area 0
       st4(rho + 4 * j, a * mu[cc].x, a * mu[cc].y, a * mu[cc].z, Real(0));
-      rh[cc] = to_velocity(sun + 4 * j);
+      if constexpr (kF64) rh[cc] = to_velocity(sun + 4 * j);
     }
     const int nh = s_nh[st];
     for (int q = tid; q < nh; q += NT) {
@@ -528,7 +662,7 @@ __global__ void __launch_bounds__(NT, adjoint_min_blocks<Real, NT>())
       const V4<Real> c = ld4(rho + 4 * j);
       const Real a = scale(harea[q]);
       st4(rho + 4 * j, a * c.x, a * c.y, a * c.z, Real(0));
-      to_velocity(sun + 4 * j);
+      if constexpr (kF64) to_velocity(sun + 4 * j);
     }
   };
   int timeout = 0;
@@ -585,6 +719,11 @@ __global__ void __launch_bounds__(NT, adjoint_min_blocks<Real, NT>())
       load_area(tile_of(k + 1));
       load_mu(tile_of(k + 1));
     }
+    int g0 = 0, g1 = 0;  // the tile's gauge cells
+    if (A.gstep >= 0) {
+      g0 = A.gauges.tile_first[tile];
+      g1 = A.gauges.tile_first[tile + 1];
+    }
     int lo = 0, hi = TC, n_faces = nrec;
     if constexpr (Parts) {
       part_of(k, lo, hi);
@@ -611,7 +750,7 @@ __global__ void __launch_bounds__(NT, adjoint_min_blocks<Real, NT>())
         const int ia = (-1 - a) & (TC - 1);
         const V4<Real> UA = ld4(sun + 4 * ia);
         const V4<Real> RA = ld4(rho + 4 * ia);
-        face_vjp<Real, true>(UA, UA, nx, ny, len, num, RA.x, RA.y, RA.z, Real(0), Real(0), Real(0),
+        face_vjp<true>(UA, UA, nx, ny, len, num, RA.x, RA.y, RA.z, Real(0), Real(0), Real(0),
                              gA, gB);
         st4(slots + 4 * slot_pad<TC>(-1 - a), gA[0], gA[1], gA[2], gA[3]);
         continue;
@@ -622,7 +761,7 @@ __global__ void __launch_bounds__(NT, adjoint_min_blocks<Real, NT>())
       const V4<Real> UB = ld4(sun + 4 * ib);
       const V4<Real> RA = ld4(rho + 4 * ia);
       const V4<Real> RB = ld4(rho + 4 * ib);
-      face_vjp<Real, false>(UA, UB, nx, ny, len, num, RA.x, RA.y, RA.z, RB.x, RB.y, RB.z, gA, gB);
+      face_vjp<false>(UA, UB, nx, ny, len, num, RA.x, RA.y, RA.z, RB.x, RB.y, RB.z, gA, gB);
       if (a < 0) st4(slots + 4 * slot_pad<TC>(-1 - a), gA[0], gA[1], gA[2], gA[3]);
       if (b < 0) st4(slots + 4 * slot_pad<TC>(-1 - b), gB[0], gB[1], gB[2], gB[3]);
     }
@@ -643,14 +782,25 @@ __global__ void __launch_bounds__(NT, adjoint_min_blocks<Real, NT>())
       const V4<Real> f1 = ld4(slots + 4 * (TC + kSlotPad + j));
       const V4<Real> f2 = ld4(slots + 4 * (2 * (TC + kSlotPad) + j));
       const V4<Real> c = ld4(sun + 4 * j);
-      const Real su = f0.y + f1.y + f2.y, sv = f0.z + f1.z + f2.z, r = rh[cc];
-      Real lh = mu[cc].x + (f0.x + f1.x + f2.x - r * fma_rn(su, c.y, sv * c.z));
-      Real lx = fma_rn(su, r, mu[cc].y), ly = fma_rn(sv, r, mu[cc].z);
-      const Real lz = mu[cc].w + (f0.w + f1.w + f2.w);
+      Real lh, lx, ly, qx = c.y, qy = c.z;
+      if constexpr (kF64) {  // velocities' derivatives back to (hu, hv)
+        const Real su = f0.y + f1.y + f2.y, sv = f0.z + f1.z + f2.z, r = rh[cc];
+        lh = mu[cc].x + (f0.x + f1.x + f2.x - r * fma_rn(su, c.y, sv * c.z));
+        lx = fma_rn(su, r, mu[cc].y);
+        ly = fma_rn(sv, r, mu[cc].z);
+        qx = c.x * c.y;
+        qy = c.x * c.z;
+      } else {
+        lh = mu[cc].x + f0.x + f1.x + f2.x;
+        lx = mu[cc].y + f0.y + f1.y + f2.y;
+        ly = mu[cc].z + f0.z + f1.z + f2.z;
+      }
+      const Real lz = mu[cc].w + f0.w + f1.w + f2.w;
+      for (int g = g0; g < g1; ++g)
+        if (A.gauges.cells[g] == base + j) lh = add_seeds(lh, A.gauges, A.gstep, g);
       if (!A.last) {
         Real b;
-        cell_vjp<Real>(c.x, c.x * c.y, c.x * c.z, lh, lx, ly, gn2[cc], A.dt_prev, num, lh, lx, ly,
-                       b);
+        cell_vjp(c.x, qx, qy, lh, lx, ly, gn2[cc], A.dt_prev, num, lh, lx, ly, b);
         A.dgn2[base + j] = dg[cc] + b;
       }
       st4(A.mu_out + 4 * (int64_t)(base + j), lh, lx, ly, lz);
@@ -665,27 +815,15 @@ __global__ void __launch_bounds__(NT, adjoint_min_blocks<Real, NT>())
       if ((pending >> i) & 1u) mbar_wait(&bar[i], (parity_bits >> i) & 1u);
     atomicOr(A.err, kErrTimeout);
   }
-  // The last block to finish adds the gauge seeds.
-  if (A.gstep >= 0) {
-    __shared__ int s_last;
-    __syncthreads();
-    if (tid == 0) {
-      __threadfence();
-      s_last = atomicAdd(A.ticket, 1u) == gridDim.x - 1u;
-    }
-    __syncthreads();
-    if (s_last) {
-      __threadfence();
-      add_gauge_seeds(A.mu_out, A.gauges, A.gstep, tid, NT);
-      if (tid == 0) *A.ticket = 0u;
-    }
-  }
 }
 
-// Adds the gauge seeds of step k to lam (one block).
+// Adds the gauge seeds of step k to lam, one thread per distinct cell.
 template <typename Real>
 __global__ void k_inject_gauges(Real* lam, GaugeSeeds g, long long k) {
-  add_gauge_seeds(lam, g, k, threadIdx.x, blockDim.x);
+  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < g.ncells; c += gridDim.x * blockDim.x) {
+    Real* p = lam + 4 * (int64_t)g.cells[c];
+    *p = add_seeds(*p, g, k, c);
+  }
 }
 
 }  // namespace swe

@@ -286,7 +286,6 @@ struct swe_tape {
   swe::Ctl* ctl = nullptr;      // two replay control words (one per ring)
   double* partial = nullptr;    // two arrays of per-chunk mass partials
   int* err = nullptr;
-  unsigned int* ticket = nullptr;
   std::vector<double> dts;
   swe::AdjLayout adj{};
   float record_ms = 0.f, grad_ms = 0.f;
@@ -438,7 +437,6 @@ swe_status grad_t(swe_tape* t, bool seeds_gauge, int* lam_cur) {
       a.err = t->err;
       a.gauges = t->gauges;
       a.gstep = (seeds_gauge && j >= 1) ? (long long)(j - 1) : -1ll;  // lambda^j gets dL/dh^j
-      a.ticket = t->ticket;
       launch_adjoint<Real>(m, t->chunks, (int)t->nchunks, a, t->adj, st);
       cur ^= 1;
     }
@@ -524,12 +522,11 @@ swe_status grad_record(swe_state* s, int64_t n_steps, int64_t checkpoint_every,
   L.add(8 * t->N * std::max(1, t->G));  // gauge depths
   L.add(8 * t->N * std::max(1, t->G));  // gauge seeds
   L.add(4 * std::max(1, t->G));
-  L.add(4 * (3 * (size_t)t->G + 1));  // gauges by cell
+  L.add(4 * (3 * (size_t)t->G + 1 + (size_t)m->ntiles + 1));  // gauges by cell and tile
   L.add(sizeof(swe::Chunk) * chunks.size());
   L.add(2 * sizeof(swe::Ctl));
   L.add(2 * 8 * (size_t)std::max<int64_t>(1, m->nchunks));
   L.add(sizeof(int));
-  L.add(sizeof(unsigned int));
   if (!arena_alloc(t->arena, L.total)) {
     free_tape(t);
     return SWE_ENOMEM;
@@ -551,12 +548,11 @@ swe_status grad_record(swe_state* s, int64_t n_steps, int64_t checkpoint_every,
   t->gauge_dev = (double*)t->arena.take(8 * t->N * std::max(1, t->G));
   t->gseed_dev = (double*)t->arena.take(8 * t->N * std::max(1, t->G));
   t->gcells = (int32_t*)t->arena.take(4 * std::max(1, t->G));
-  int32_t* by_cell = (int32_t*)t->arena.take(4 * (3 * (size_t)t->G + 1));
+  int32_t* by_cell = (int32_t*)t->arena.take(4 * (3 * (size_t)t->G + 1 + (size_t)m->ntiles + 1));
   t->chunks = (swe::Chunk*)t->arena.take(sizeof(swe::Chunk) * chunks.size());
   t->ctl = (swe::Ctl*)t->arena.take(2 * sizeof(swe::Ctl));
   t->partial = (double*)t->arena.take(2 * 8 * (size_t)std::max<int64_t>(1, m->nchunks));
   t->err = (int*)t->arena.take(sizeof(int));
-  t->ticket = (unsigned int*)t->arena.take(sizeof(unsigned int));
   if (t->arena.overflow) {
     g_cuda_msg = "tape arena layout";
     free_tape(t);
@@ -605,12 +601,17 @@ swe_status grad_record(swe_state* s, int64_t n_steps, int64_t checkpoint_every,
       }
     first.push_back(t->G);
     const int nc = (int)cells.size();
-    t->gauges = {by_cell, by_cell + t->G, by_cell + 2 * t->G + 1, t->gseed_dev, t->G, nc};
+    std::vector<int32_t> tiles(m->ntiles + 1, 0);  // where each tile's cells start
+    for (int32_t c : cells) tiles[c / m->tile + 1] += 1;
+    for (int64_t k = 0; k < m->ntiles; ++k) tiles[k + 1] += tiles[k];
+    t->gauges = {by_cell, by_cell + t->G, by_cell + 2 * t->G + 1, by_cell + 3 * t->G + 1, t->gseed_dev,
+                 t->G, nc};
     auto put = [&](const int32_t* to, const std::vector<int32_t>& v) {
       return cuda_failed(cudaMemcpyAsync((void*)to, v.data(), 4 * v.size(), cudaMemcpyHostToDevice,
                                          m->stream));
     };
     if (put(t->gauges.cells, cells) || put(t->gauges.first, first) || put(t->gauges.index, index) ||
+        put(t->gauges.tile_first, tiles) ||
         cuda_failed(cudaStreamSynchronize(m->stream)))
       return fail(SWE_ECUDA);
   }
@@ -661,7 +662,6 @@ swe_status grad(swe_tape* t, const double* g_h, const double* g_hu, const double
   CK(cudaMemsetAsync(t->lam[0], 0, sb, st));
   CK(cudaMemsetAsync(t->lam[1], 0, sb, st));
   CK(cudaMemsetAsync(t->err, 0, sizeof(int), st));
-  CK(cudaMemsetAsync(t->ticket, 0, sizeof(unsigned int), st));
   const double* seeds[3] = {g_h, g_hu, g_hv};
   for (int c = 0; c < 3; ++c) {
     if (!seeds[c]) continue;
