@@ -320,7 +320,7 @@ typedef struct swe_tape swe_tape;
  * gauge_cells[j] (caller indices, repeats allowed) after every step into
  * gauge_h[k * n_gauges + j] for step k = 0 .. n_steps-1 (host, may be NULL),
  * the state every checkpoint_every steps, and the K - 1 inner states of the
- * last segment (device memory: about ceil(n_steps / K) + 3K states,
+ * last three segments (device memory: about ceil(n_steps / K) + 3K states,
  * K = checkpoint_every; K = 1 keeps every state and swe_grad then recomputes
  * nothing). The state is
  * left at step n_steps. Synchronises. Returns SWE_ENAN / SWE_EDRY if a step
@@ -334,7 +334,7 @@ swe_status swe_grad_record(swe_state* state, int64_t n_steps, int64_t checkpoint
  * [n_tris each]; g_gauge = dL/d gauge_h [n_steps * n_gauges]. Outputs (host,
  * caller order, any may be NULL): dL/dh, dL/dhu, dL/dhv of the initial state,
  * dL/dz, dL/dn (n >= 0 assumed). Recomputes each segment of checkpoint_every
- * steps but the last from its checkpoint; returns SWE_ESTATE if a recomputed
+ * steps whose inner states the tape does not hold from its checkpoint; returns SWE_ESTATE if a recomputed
  * step did not reproduce the recorded dt. Synchronises. */
 swe_status swe_grad(swe_tape* tape, const double* g_h, const double* g_hu, const double* g_hv,
                     const double* g_gauge, double* d_h0, double* d_hu0, double* d_hv0, double* d_z,
