@@ -112,7 +112,14 @@ def tune(cases, precision: str = "f32", *, candidates=CANDIDATES, steps: int = 3
     "sec_per_step", "cached", "trials": [...]}.
     """
     import torch
-    n_cells = key_cells if key_cells is not None else sum(c.mesh.n_tris for c in cases)
+    cases = list(cases)
+    sampled = sum(c.mesh.n_tris for c in cases)
+    n_cells = key_cells if key_cells is not None else sampled
+    if len(cases) > 1:
+        # A sample of a large ensemble is repeated until its blocks walk as many
+        # tiles as the whole's: ensembles of a few million cells run in one wave
+        # of blocks, larger ones in three, and the shapes rank differently.
+        cases = cases * max(1, math.ceil(min(n_cells, 9_500_000) / sampled))
     n_scen = key_scenarios if key_scenarios is not None else len(cases)
     name = torch.cuda.get_device_name(torch.cuda.current_device())
     key = problem_key(name, precision, n_cells, n_scen)

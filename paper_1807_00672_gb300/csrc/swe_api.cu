@@ -288,7 +288,7 @@ constexpr int64_t kSmallTileCells = 6000000;
 constexpr int kDefaultTileF64 = 256;
 // No mesh above this many cells fits the resident kernel (the chip's shared
 // memory holds about 330,000 FP32 or 175,000 FP64 cells).
-constexpr int64_t kResidentCells = 400000;
+constexpr int64_t kResidentCellsF32 = 340000, kResidentCellsF64 = 180000;
 // Several scenarios: up to kEnsembleWaves waves of work chunks, of at least
 // kWaveTiles tiles each. More waves balance uneven scenarios better, but each
 // block pays its first copies again: 32 scenarios of 2.3M cells (9.7 tiles of
@@ -779,23 +779,19 @@ swe_status create_batch(int32_t n, const double* const* xy, const int64_t* n_nod
   const int tile = p.tile;
   // The resident kernel runs meshes whose shape the caller left to the
   // library, if they fit in the chip's shared memory.
-  const bool keep_edges = default_shape && autok && !ghost && all_tris <= kResidentCells;
+  const bool keep_edges = default_shape && autok && !ghost &&
+                          all_tris <= (p.precision == SWE_F64 ? kResidentCellsF64 : kResidentCellsF32);
 
   // Host-side construction and validation first (scenarios on parallel host
   // threads): no device is touched for an invalid mesh.
   std::vector<swe::HostMesh> hm(n);
   std::vector<int> rc(n, 0);
-  {
+  auto over_scenarios = [&](auto&& body) {  // on parallel host threads
     const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
     const int nthr = (int)std::min<unsigned>((unsigned)n, std::min(16u, hw));
     std::atomic<int> next{0};
     auto work = [&]() {
-      for (int i = next++; i < n; i = next++)
-        rc[i] = swe::build_host_mesh(xy[i], n_nodes[i], tri[i], n_tris[i], p.order,
-                                     kernel == SWE_KERNEL_TILED ? tile : 0,
-                                     kernel == SWE_KERNEL_EDGE, hm[i],
-                                     kernel == SWE_KERNEL_TILED && p.precision == SWE_F32 && !keep_edges,
-                                     keep_edges);
+      for (int i = next++; i < n; i = next++) body(i);
     };
     std::vector<std::thread> pool;
     try {  // the calling thread takes every scenario no worker takes
@@ -804,7 +800,14 @@ swe_status create_batch(int32_t n, const double* const* xy, const int64_t* n_nod
     }
     work();
     for (auto& t : pool) t.join();
-  }
+  };
+  over_scenarios([&](int i) {
+    rc[i] = swe::build_host_mesh(xy[i], n_nodes[i], tri[i], n_tris[i], p.order,
+                                 kernel == SWE_KERNEL_TILED ? tile : 0, kernel == SWE_KERNEL_EDGE,
+                                 hm[i],
+                                 kernel == SWE_KERNEL_TILED && p.precision == SWE_F32 && !keep_edges,
+                                 keep_edges);
+  });
   for (int i = 0; i < n; ++i) {
     if (rc[i] == -2) return SWE_EMESH;
     if (rc[i] != 0) return SWE_EINVAL;
@@ -925,7 +928,12 @@ swe_status create_batch(int32_t n, const double* const* xy, const int64_t* n_nod
   // The bank order of the FP32 tiles was left out where the resident kernel
   // might step the mesh.
   if (keep_edges && m->res.nblocks == 0 && kernel == SWE_KERNEL_TILED && p.precision == SWE_F32)
-    for (swe::HostMesh& h : hm) swe::order_records_for_banks(h);
+    over_scenarios([&](int i) {
+      try {
+        swe::order_records_for_banks(hm[i]);
+      } catch (...) {  // no host memory: the records stay in their order, same results
+      }
+    });
 
   // Device layout.
   const int64_t T = m->T, Tp = m->Tp, E = m->E, R = recs, H = halos;
