@@ -599,12 +599,12 @@ def ensemble_error(cases, mesh, st, steps, every=16):
     return res
 
 
-# Algorithmic bytes per cell of one adjoint step: reads U^n (h, hu, hv, z),
-# U^{n+1} (h, hu, hv), lambda^{n+1} (4 words), area, g n^2 and the running
-# dL/d(g n^2), the edge geometry and endpoints once (1.5 edges per cell);
-# writes lambda^n (4 words) and dL/d(g n^2): 23.5 words + 12 bytes.
+# Algorithmic bytes per cell of one adjoint step: reads U^n (h, hu, hv, z), mu
+# of the step (4 words), area, g n^2 and the running dL/d(g n^2), the edge
+# geometry and endpoints once (1.5 edges per cell); writes mu of the step
+# before (4 words) and dL/d(g n^2): 20.5 words + 12 bytes.
 def adjoint_bytes_per_cell(word: int) -> float:
-    return 23.5 * word + 12.0
+    return 20.5 * word + 12.0
 
 
 def adjoint_leg(args, stream, errors):
