@@ -113,3 +113,34 @@ def test_many_small_sub_domains_on_one_gpu():
         for a, b in zip(run.fields(), ref.fields()):
             assert np.array_equal(a, b), prec
         run.close()
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+def test_a_dry_sub_domain_hands_out_an_infinite_time_step(prec):
+    """The CFL step of a sub-domain with no wet cell of its own is +inf (not
+    NaN, which a minimum over the sub-domains need not drop), on the device
+    and on the host, at its initialisation and after steps; the minimum with
+    a wet sub-domain's step is that step."""
+    torch = pytest.importorskip("torch")
+    ensure_built()
+    case = inputs.random_flow_case(nx=12, ny=9, seed=5)
+    ghost = np.zeros(case.mesh.n_tris, np.uint8)
+    ghost[:7] = 1
+    mesh = swe.Mesh.part(case.mesh.xy, case.mesh.tri, ghost, precision=prec)
+    dry = [np.zeros(mesh.T) for _ in range(3)]
+    st = swe.State(mesh, *dry, case.z, case.n)
+    wet = swe.State(mesh, case.h, case.hu, case.hv, case.z, case.n)
+    dts = torch.zeros(2, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    for _ in range(2):
+        st.dt_device(dts[:1].data_ptr())
+        wet.dt_device(dts[1:].data_ptr())
+        assert st.next_dt() == np.inf
+        wet.sync()
+        assert dts[0].item() == np.inf and 0.0 < dts[1].item() < np.inf
+        want = wet.next_dt()
+        for s in (st, wet):
+            s.set_dt_min_device(dts.data_ptr(), 2)
+            assert s.next_dt() == want
+            s.run(1)
+    assert st.info()["err"] == 0 and np.all(st.fields()[0] == 0.0)
