@@ -323,6 +323,7 @@ __global__ void __launch_bounds__(res_max_threads<Real, CH>(), 1)
     top = warp_max_bits(top);
     err |= (int)__reduce_or_sync(0xffffffffu, bad);
     if (top == 0ull) err |= kErrDry;
+    err |= rate_error(__longlong_as_double((long long)top));
     if (err) {
       done = 1;
       dt_now = 0.0;

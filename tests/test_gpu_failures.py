@@ -88,3 +88,23 @@ def test_negative_input_depths_are_clipped_and_counted(kernel):
     errs, (h, _, _) = field_errors(st, ref)
     assert max(errs.values()) <= 1e-11, errs
     assert np.all(h >= 0.0)
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("kernel", ["tiled", "edge", "auto"])
+def test_a_rate_that_overflows_is_an_error(kernel, prec):
+    """Momentum whose square overflows, in a dry cell that the first step
+    wets: the CFL rate is infinite and the next time step would be 0, at this
+    and every later step. The step latches SWE_ENAN; advance ends with it."""
+    ensure_built()
+    case = inputs.random_flow_case(nx=37, ny=23, seed=41)
+    assert case.h[100] == 0.0
+    case.hu[100] = 1e30 if prec == "f32" else 1e200
+    case.n[:] = 0.0
+    mesh = swe.Mesh(case.mesh.xy, case.mesh.tri, precision=prec, kernel=kernel)
+    for call in (lambda st: st.run(30), lambda st: st.advance(1e3)):
+        st = swe.State(mesh, case.h, case.hu, case.hv, case.z, case.n)
+        with pytest.raises(swe.SweError) as ei:
+            call(st)
+        assert ei.value.status == swe.SWE_ENAN
+        assert st.info()["err"] == 1
