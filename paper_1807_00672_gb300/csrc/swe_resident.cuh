@@ -23,8 +23,15 @@
 // A block publishes epoch e + 2 only after it has read every slot of epoch
 // e + 1, and a block writes its slot of epoch e + 1 only after its faces have
 // read every word of epoch e and its control warp every slot of epoch e.
-// Epochs grow over the life of a state (Ctl resets do not touch them), so no
-// word of an earlier launch can be taken for a new one.
+// Epochs grow over the life of a state (Ctl resets do not touch them): every
+// launch advances the epoch past every word it could publish, whether it
+// steps, stops or gives up (pass_entry), so no word of an earlier launch can
+// be taken for a new one.
+//
+// A block that gives up may do so, and set the stop flag, before others have
+// started: one thread of each block reads the flag and the epoch, so a block
+// goes on or leaves as a whole. A launch in which a block gave up cannot end
+// well for the scenario (its rate never comes), whoever still joined it.
 #pragma once
 
 #include "swe_kernels.cuh"
@@ -111,14 +118,30 @@ __device__ __forceinline__ void ld_word(const void* p, unsigned long long& a, un
       : "memory");
 }
 
+// Whether a block of the scenario has given up.
+__device__ __forceinline__ bool timed_out(const Ctl* ctl) {
+  return *(const volatile int*)&ctl->err & kErrTimeout;
+}
+
+// One thread of each block calls this once the block has read the epoch of
+// the launch. The last of the scenario's nblocks blocks advances it to `next`,
+// which nothing but the next launch reads.
+__device__ __forceinline__ void pass_entry(Ctl* ctl, uint32_t* epoch, uint32_t next, int nblocks) {
+  __threadfence();
+  if (atomicAdd(&ctl->ticket, 1u) != (unsigned)nblocks - 1u) return;
+  __threadfence();
+  ctl->ticket = 0u;
+  *epoch = next;
+}
+
 // Polls a word until the epoch in its last 4 bytes is e; false after `limit`
-// reads, or once another block has latched an error.
+// reads, or once another block has given up.
 __device__ __forceinline__ bool poll_word(const void* p, uint32_t e, uint32_t limit, const Ctl* ctl,
                                           unsigned long long& a, unsigned long long& b) {
   for (uint32_t i = 0; i < limit; ++i) {
     ld_word(p, a, b);
     if ((uint32_t)(b >> 32) == e) return true;
-    if ((i & 1023u) == 1023u && *(const volatile int*)&ctl->err) return false;
+    if ((i & 1023u) == 1023u && timed_out(ctl)) return false;
   }
   return false;
 }
@@ -153,7 +176,7 @@ __device__ __forceinline__ bool read_cell(const unsigned char* w, uint32_t e, ui
     ld_word(w, a, b);
     ld_word(w + 16, d, f);
     ok = (uint32_t)(b >> 32) == e && (uint32_t)(f >> 32) == e;
-    if (ok || ((i & 1023u) == 1023u && *(const volatile int*)&ctl->err)) break;
+    if (ok || ((i & 1023u) == 1023u && timed_out(ctl))) break;
   }
   c.x = __longlong_as_double((long long)a);
   c.y = __longlong_as_double((long long)((b & 0xffffffffull) | f << 32));
@@ -199,7 +222,8 @@ __global__ void __launch_bounds__(res_max_threads<Real, CH>(), 1)
   __shared__ unsigned long long s_wrate[32];
   __shared__ unsigned s_wbad[32], s_count;
   __shared__ Real s_dt;
-  __shared__ int s_stop, s_fail;
+  __shared__ int s_stop, s_fail, s_leave;
+  __shared__ uint32_t s_epoch;
   Real* sc = reinterpret_cast<Real*>(smem);
   const int4* srec = reinterpret_cast<const int4*>(smem + L.off_rec);
   uint32_t* sside = reinterpret_cast<uint32_t*>(smem + L.off_rec);
@@ -219,11 +243,20 @@ __global__ void __launch_bounds__(res_max_threads<Real, CH>(), 1)
 
   const ResBlock blk = P.blocks[blockIdx.x];
   Ctl* ctl = s.ctl + blk.scen;
-  if (ctl->done) return;  // nothing writes it before every block has passed here
   const int tid = threadIdx.x, nthr = blockDim.x, nct = nthr - 32, lane = tid & 31;
   const bool control = tid >= nct;
-  const int cur = ctl->cur;
-  const uint32_t e0 = P.epoch[blk.scen] + 1u;  // epoch of the state at entry
+  const int cur = ctl->cur;  // written only once every block has stepped
+  if (tid == 0) {
+    s_epoch = P.epoch[blk.scen] + 1u;
+    s_leave = *(const volatile int*)&ctl->done | (int)timed_out(ctl);
+  }
+  __syncthreads();
+  const uint32_t e0 = s_epoch;  // epoch of the state at entry
+  const uint32_t e_next = e0 + (uint32_t)n_steps + 1u;
+  if (s_leave) {
+    if (tid == 0) pass_entry(ctl, P.epoch + blk.scen, e_next, blk.nblocks);
+    return;
+  }
   const uint32_t limit = num.wait_rounds >= 0xffffffffu / kPollsPerRound
                              ? 0xffffffffu
                              : num.wait_rounds * kPollsPerRound;
@@ -311,7 +344,7 @@ __global__ void __launch_bounds__(res_max_threads<Real, CH>(), 1)
         ok = true;
 #pragma unroll
         for (int q = 0; q < kBatch; ++q) ok = ok && (uint32_t)(b[q] >> 32) == e;
-        if (!ok && (n & 1023u) == 1023u && *(const volatile int*)&ctl->err) break;
+        if (!ok && (n & 1023u) == 1023u && timed_out(ctl)) break;
       }
 #pragma unroll
       for (int q = 0; q < kBatch; ++q) {
@@ -351,6 +384,8 @@ __global__ void __launch_bounds__(res_max_threads<Real, CH>(), 1)
           if (done) s_stop = 1;
           if (!ok) s_fail = 1;
         }
+      } else if (lane == 0) {  // idle otherwise
+        pass_entry(ctl, P.epoch + blk.scen, e_next, blk.nblocks);
       }
     } else {
       // A warp's 32 records together: its lanes meet again after the polls,
@@ -495,8 +530,26 @@ __global__ void __launch_bounds__(res_max_threads<Real, CH>(), 1)
   // After the last step its rate gives the next dt (the scenario's first
   // block needs it); a step that ended the run has set the clock already.
   if (!timeout && k == n_steps && control && blk.first) timeout = !next_clock(e0 + (uint32_t)k);
-  // State after the step(s): the other buffer (the one read at entry may
-  // still be read by a block that has not started).
+  if (control && lane == 0) {
+    if (timeout) {
+      atomicOr(&ctl->err, kErrTimeout);
+      ctl->done = 1;
+      ctl->dt = 0.0;
+      ctl->dt_cfl = 0.0;
+    } else if (blk.first) {
+      ctl->t = t;
+      ctl->dt = dt_now;
+      ctl->dt_cfl = dt_cfl;
+      ctl->dt_last = dt_last;
+      ctl->steps += taken;
+      if (taken > 0) ctl->cur = cur ^ 1;
+      ctl->clamped = clamped;
+      if (err) atomicOr(&ctl->err, err);
+      if (done) ctl->done = 1;
+    }
+  }
+  // State after the step(s), into the other buffer: until the buffer number
+  // changes, the one read at entry is the state.
   if (!timeout && k > 0) {
     Real* oh = cur ? s.h[0] : s.h[1];
     Real* ohu = cur ? s.hu[0] : s.hu[1];
@@ -521,25 +574,6 @@ __global__ void __launch_bounds__(res_max_threads<Real, CH>(), 1)
   }
   const int wneg = __reduce_add_sync(0xffffffffu, neg);
   if (lane == 0 && wneg) atomicAdd((unsigned long long*)&ctl->neg, (unsigned long long)wneg);
-  if (timeout) {
-    if (lane == 0) {
-      atomicOr(&ctl->err, kErrTimeout);
-      ctl->done = 1;
-      ctl->dt = 0.0;
-      ctl->dt_cfl = 0.0;
-    }
-  } else if (control && lane == 0 && blk.first) {
-    ctl->t = t;
-    ctl->dt = dt_now;
-    ctl->dt_cfl = dt_cfl;
-    ctl->dt_last = dt_last;
-    ctl->steps += taken;
-    if (taken > 0) ctl->cur = cur ^ 1;
-    ctl->clamped = clamped;
-    if (err) atomicOr(&ctl->err, err);
-    if (done) ctl->done = 1;
-  }
-  if (control && lane == 0 && blk.first) P.epoch[blk.scen] = e0 + (uint32_t)n_steps + 1u;
 }
 
 }  // namespace swe

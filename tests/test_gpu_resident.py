@@ -4,6 +4,10 @@ are those of the one-step tiled kernel (the same arithmetic per face and
 cell, and the same dt sequence): equal bit for bit, over sizes from one cell
 to the largest that fits, both precisions, every cell order, ensembles, the
 depth residual, any split of a run into calls, and end times."""
+import os
+import shutil
+import subprocess
+
 import numpy as np
 import pytest
 
@@ -158,3 +162,42 @@ def test_errors_are_latched(prec):
     st = pair(ok, "f64")[0]
     st.run(20)
     assert max(field_errors(st, ref)[0].values()) <= 1e-11
+
+
+def test_every_launch_advances_the_epoch(tmp_path):
+    """pass_entry alone (tests/resident_entry_check.cu): the epoch a launch's
+    blocks read, and the one it leaves, in whatever order they start."""
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    exe = str(tmp_path / "resident_entry_check")
+    subprocess.run([nvcc, "-O3", "-std=c++17", "-gencode", "arch=compute_103a,code=sm_103a", "-o", exe,
+                    os.path.join(os.path.dirname(os.path.abspath(__file__)), "resident_entry_check.cu")],
+                   check=True)
+    r = subprocess.run([exe], capture_output=True, text=True)
+    assert r.returncode == 0 and r.stdout.strip() == "ok", r.stdout
+
+
+@pytest.mark.parametrize("prec,order", [("f64", "morton"), ("f32", "morton"), ("f32", "rcm")])
+@pytest.mark.parametrize("nx,ny", [(3, 2), (37, 23), (150, 75)])
+def test_launches_that_give_up_leave_the_state_alone(prec, order, nx, ny):
+    """Waits that run out at once: every kind of call reports SWE_ETIMEOUT,
+    again after the state is set anew (which clears the error), takes no step
+    and leaves the fields as they were."""
+    ensure_built()
+    case = inputs.random_flow_case(nx=nx, ny=ny, seed=41)
+    mesh = swe.Mesh(case.mesh.xy, case.mesh.tri, precision=prec, order=order, wait_rounds=-1)
+    st = swe.State(mesh, case.h, case.hu, case.hv, case.z, case.n)
+    before = st.fields()
+    dt = st.next_dt()
+    for call in (lambda: st.run(5), lambda: st.step(), lambda: st.advance(1.0), lambda: st.run(5000)):
+        for _ in range(2):
+            with pytest.raises(swe.SweError) as ei:
+                call()
+            assert ei.value.status == swe.SWE_ETIMEOUT
+        assert st.info() == dict(steps=0, neg=0, err=4)
+        after = [np.empty(mesh.T) for _ in range(3)]
+        with pytest.raises(swe.SweError):  # copies out all the same
+            st.copy_out(*after)
+        for a, b in zip(after, before):
+            assert np.array_equal(a, b)
+        st.set(case.h, case.hu, case.hv)
+        assert st.info()["err"] == 0 and st.next_dt() == dt
