@@ -101,9 +101,11 @@ typedef struct {
                                 autotuner. 1 and 2 apply to FP32 meshes with 2 stages whose
                                 halo lists fit one entry per thread, and are ignored
                                 otherwise. Results are identical. */
-  int32_t wait_rounds;       /* bounded device waits of SWE_KERNEL_TILED steps (a block waiting
-                                for its tile copies) give up after this many rounds of at most
-                                20 us and latch SWE_ETIMEOUT: 0 = default (50,000 rounds,
+  int32_t wait_rounds;       /* bounded device waits (of SWE_KERNEL_TILED steps: a block waiting
+                                for its tile copies; of meshes that stay on chip: a block
+                                waiting for another block's cells or CFL rate) give up after
+                                this many rounds of at most 20 us, on chip after about 45 ms
+                                more, and latch SWE_ETIMEOUT: 0 = default (50,000 rounds,
                                 about a second); n > 0 = n rounds; -1 = give up at once, so
                                 every step of the mesh ends with SWE_ETIMEOUT (a hook for
                                 testing the timeout path: copies already in flight are still

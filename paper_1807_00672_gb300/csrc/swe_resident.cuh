@@ -204,8 +204,16 @@ __device__ __forceinline__ unsigned long long warp_max_bits(double v) {
 template <typename Real, bool CH>
 constexpr int res_max_threads() { return sizeof(Real) == 8 ? 544 : CH ? 800 : 1024; }
 
-// Polls per round of swe_params.wait_rounds (a round is at most about 20 us).
-constexpr uint32_t kPollsPerRound = 32;
+// Polls per round of swe_params.wait_rounds (a round is at most about 20 us),
+// on top of kLeastPolls (about 45 ms). A block's own copies take microseconds,
+// which one round covers; here it waits for other blocks, which may start tens
+// of microseconds apart and take a step of up to 50.
+constexpr uint32_t kPollsPerRound = 32, kLeastPolls = 1u << 16;
+__device__ __forceinline__ uint32_t most_polls(uint32_t rounds) {
+  if (rounds == 0u) return 0u;  // the caller asked for no wait at all
+  return rounds < (0xffffffffu - kLeastPolls) / kPollsPerRound ? kLeastPolls + rounds * kPollsPerRound
+                                                              : 0xffffffffu;
+}
 
 // Up to n_steps steps of every scenario (fewer where one reaches its end time
 // or an error). The last warp of a block is its control warp: while the
@@ -257,9 +265,7 @@ __global__ void __launch_bounds__(res_max_threads<Real, CH>(), 1)
     if (tid == 0) pass_entry(ctl, P.epoch + blk.scen, e_next, blk.nblocks);
     return;
   }
-  const uint32_t limit = num.wait_rounds >= 0xffffffffu / kPollsPerRound
-                             ? 0xffffffffu
-                             : num.wait_rounds * kPollsPerRound;
+  const uint32_t limit = most_polls(num.wait_rounds);
   auto pub_word = [&](uint32_t e, int p) {
     return P.xbuf + ((size_t)(e & 1u) * P.npub + p) * pub_bytes<Real>();
   };

@@ -7,6 +7,7 @@ depth residual, any split of a run into calls, and end times."""
 import os
 import shutil
 import subprocess
+import threading
 
 import numpy as np
 import pytest
@@ -201,3 +202,62 @@ def test_launches_that_give_up_leave_the_state_alone(prec, order, nx, ny):
             assert np.array_equal(a, b)
         st.set(case.h, case.hu, case.hv)
         assert st.info()["err"] == 0 and st.next_dt() == dt
+
+
+@pytest.mark.parametrize("prec,nx,ny", [("f64", 50, 25), ("f64", 400, 205), ("f32", 71, 71),
+                                        ("f32", 560, 280)])
+def test_the_shortest_waits_do_not_end_a_valid_run(prec, nx, ny):
+    """wait_rounds = 1: blocks that start apart, or wait for the slowest of a
+    step, stay far below the limit, launch after launch."""
+    case = small_case(nx, ny, 7)
+    ref = pair(case, prec)[1]
+    ref.run(12)
+    mesh = swe.Mesh(case.mesh.xy, case.mesh.tri, precision=prec, wait_rounds=1)
+    st = swe.State(mesh, case.h, case.hu, case.hv, case.z, case.n)
+    for _ in range(30):
+        st.set(case.h, case.hu, case.hv)
+        for n in (1, 2, 9):
+            st.run(n, sync=False)
+        assert_same(st, ref)
+
+
+def test_states_on_streams_and_threads_of_their_own():
+    """Resident launches of several states at once, small ones that share the
+    SMs and large ones that take the chip in turn, from a thread each: the
+    results are those of the same run alone."""
+    ensure_built()
+    jobs = [(small_case(nx, ny, 11 + i), prec)
+            for i, (prec, nx, ny) in enumerate([("f32", 35, 30), ("f64", 25, 20), ("f32", 400, 350),
+                                                ("f64", 300, 200), ("f32", 90, 60), ("f64", 60, 40)])]
+
+    def work(job, n):
+        case, prec = job
+        mesh = swe.Mesh(case.mesh.xy, case.mesh.tri, precision=prec)
+        st = swe.State(mesh, case.h, case.hu, case.hv, case.z, case.n)
+        out = []
+        for _ in range(n):
+            st.set(case.h, case.hu, case.hv)
+            for k in (1, 5, 40):
+                st.run(k, sync=False)
+            st.advance(st.t + 3.0 * st.next_dt())
+            out.append((*st.fields(), st.t))
+        st.close()
+        mesh.close()
+        return out
+
+    want = [work(job, 1)[0] for job in jobs]
+    errors = []
+
+    def worker(i):
+        try:
+            for got in work(jobs[i], 12):
+                assert all(np.array_equal(a, b) for a, b in zip(got, want[i])), i
+        except Exception as e:  # noqa: BLE001
+            errors.append((i, e))
+
+    threads = [threading.Thread(target=worker, args=(i,)) for i in range(len(jobs))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
