@@ -24,3 +24,14 @@ def test_fp64_functions_over_all_exponents(tmp_path):
     assert err["sqrt"] <= 1.0, err
     assert err["icbrt"] <= 4.0, err
     assert err["special"] == 0, err
+
+
+def test_square_roots_are_correctly_rounded(tmp_path):
+    """The FP64 path's square root is IEEE's, bit for bit, at the arguments
+    whose roots are hardest to round too (tests/fp64_sqrt_check.cu)."""
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    exe = str(tmp_path / "fp64_sqrt_check")
+    subprocess.run([nvcc, "-O3", "-std=c++17", "-gencode", "arch=compute_103a,code=sm_103a",
+                    "-o", exe, os.path.join(HERE, "fp64_sqrt_check.cu")], check=True)
+    out = subprocess.run([exe], check=True, capture_output=True, text=True).stdout
+    assert out.strip() == "differ 0", out
