@@ -53,10 +53,11 @@ __device__ __forceinline__ double twice(double x, bool pos) {
 }
 
 // dL/dU* of one cell from its post-step state (h1, q1x, q1y) and lambda:
-// mu (3 values) and the derivative with respect to its g n^2.
-__device__ __forceinline__ void cell_vjp(float h1, float q1x, float q1y, float lh, float lx, float ly,
-                                         float gn2, float dt, const Num& num, float& mh, float& mx,
-                                         float& my, float& bgn2) {
+// mu (3 values) and the derivative with respect to its g n^2. r1: 1 / h1 of a
+// wet cell, which the FP64 form takes (FP32 divides).
+__device__ __forceinline__ void cell_vjp(float h1, float q1x, float q1y, float, float lh, float lx,
+                                         float ly, float gn2, float dt, const Num& num, float& mh,
+                                         float& mx, float& my, float& bgn2) {
   using O = Ops<float>;
   const float zero = 0.0f;
   if (O::wet(h1, num)) {
@@ -81,9 +82,9 @@ __device__ __forceinline__ void cell_vjp(float h1, float q1x, float q1y, float l
 
 // FP64: fewer FP64 instructions; the last output is left 0 where g n^2 is 0
 // (it only enters dL/dn, multiplied by n).
-__device__ __forceinline__ void cell_vjp(double h1, double q1x, double q1y, double lh, double lx,
-                                         double ly, double gn2, double dt, const Num& num, double& mh,
-                                         double& mx, double& my, double& bgn2) {
+__device__ __forceinline__ void cell_vjp(double h1, double q1x, double q1y, double r1, double lh,
+                                         double lx, double ly, double gn2, double dt, const Num& num,
+                                         double& mh, double& mx, double& my, double& bgn2) {
   using O = Ops<double>;
   const double zero = 0.0;
   mh = lh;
@@ -95,9 +96,7 @@ __device__ __forceinline__ void cell_vjp(double h1, double q1x, double q1y, doub
   my = ly;
   if (!above0(gn2)) return;
   const double q1n = O::sqrt_(fma_rn(q1x, q1x, q1y * q1y));
-  const double y = icbrt_nr(h1), y2 = mul_rn(y, y);  // h^{-1/3}
-  const double rh = mul_rn(y2, y);                   // 1 / h
-  const double ch = mul_rn(dt, mul_rn(mul_rn(y2, y2), rh));
+  const double ch = mul_rn(dt, O::pow_m73(h1));
   const double c = ch * gn2;
   const double cq = c * q1n;        // (d - 1) / d
   const double rd = 1.0 - cq;   // 1 / d
@@ -105,7 +104,7 @@ __device__ __forceinline__ void cell_vjp(double h1, double q1x, double q1y, doub
   const double k = above0(q1n) ? O::div(c * ql, q1n) : zero;
   mx = rd * fma_rn(-k, q1x, lx);
   my = rd * fma_rn(-k, q1y, ly);
-  mh = fma_rn((7.0 / 3.0) * (cq * rh), ql, lh);
+  mh = fma_rn((7.0 / 3.0) * (cq * r1), ql, lh);
   bgn2 = -(q1n * ch) * ql;
 }
 
@@ -467,7 +466,8 @@ __global__ void __launch_bounds__(256)
        i += (int64_t)gridDim.x * blockDim.x) {
     const V4<Real> c = ld4(u1 + 4 * i), l = ld4(lam + 4 * i);
     Real mh, mx, my, b;
-    cell_vjp(c.x, c.y, c.z, l.x, l.y, l.z, gn2[i], dt, num, mh, mx, my, b);
+    const Real r1 = sizeof(Real) == 8 && Ops<Real>::wet(c.x, num) ? Ops<Real>::rcp(c.x) : Real(0);
+    cell_vjp(c.x, c.y, c.z, r1, l.x, l.y, l.z, gn2[i], dt, num, mh, mx, my, b);
     st4(lam + 4 * i, mh, mx, my, l.w);
     dgn2[i] = b;
   }
@@ -617,7 +617,9 @@ __global__ void __launch_bounds__(NT, adjoint_min_blocks<Real, NT>())
   // load_mu filled, and the halo cells this thread gathered (gather_halo's
   // assignment, so no barrier is needed after its own copies land).
   V4<Real> mu[CPT];
-  Real rh[CPT];  // 1 / h of a wet cell, else 0
+  // FP64: 1 / h of a wet cell, else 0, and (hu, hv), which the staged cells
+  // lose to their velocities (h u would differ from hu by two roundings)
+  Real rh[CPT], mqx[CPT], mqy[CPT];
   auto phase_a = [&](int st, int k) {
     const int tile = tile_of(k);
     if constexpr (Parts) {  // the part's records
@@ -654,7 +656,11 @@ __global__ void __launch_bounds__(NT, adjoint_min_blocks<Real, NT>())
       mu[cc] = nmu[cc];
       const Real a = j < nc ? scale(nar[cc]) : Real(0);  // padding: area 0
       st4(rho + 4 * j, a * mu[cc].x, a * mu[cc].y, a * mu[cc].z, Real(0));
-      if constexpr (kF64) rh[cc] = to_velocity(sun + 4 * j);
+      if constexpr (kF64) {
+        mqx[cc] = sun[4 * j + 1];
+        mqy[cc] = sun[4 * j + 2];
+        rh[cc] = to_velocity(sun + 4 * j);
+      }
     }
     const int nh = s_nh[st];
     for (int q = tid; q < nh; q += NT) {
@@ -788,8 +794,8 @@ __global__ void __launch_bounds__(NT, adjoint_min_blocks<Real, NT>())
         lh = mu[cc].x + (f0.x + f1.x + f2.x - r * fma_rn(su, c.y, sv * c.z));
         lx = fma_rn(su, r, mu[cc].y);
         ly = fma_rn(sv, r, mu[cc].z);
-        qx = c.x * c.y;
-        qy = c.x * c.z;
+        qx = mqx[cc];
+        qy = mqy[cc];
       } else {
         lh = mu[cc].x + f0.x + f1.x + f2.x;
         lx = mu[cc].y + f0.y + f1.y + f2.y;
@@ -800,7 +806,8 @@ __global__ void __launch_bounds__(NT, adjoint_min_blocks<Real, NT>())
         if (A.gauges.cells[g] == base + j) lh = add_seeds(lh, A.gauges, A.gstep, g);
       if (!A.last) {
         Real b;
-        cell_vjp(c.x, qx, qy, lh, lx, ly, gn2[cc], A.dt_prev, num, lh, lx, ly, b);
+        cell_vjp(c.x, qx, qy, kF64 ? rh[cc] : Real(0), lh, lx, ly, gn2[cc], A.dt_prev, num, lh, lx, ly,
+                 b);
         A.dgn2[base + j] = dg[cc] + b;
       }
       st4(A.mu_out + 4 * (int64_t)(base + j), lh, lx, ly, lz);

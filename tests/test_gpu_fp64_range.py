@@ -35,3 +35,14 @@ def test_square_roots_are_correctly_rounded(tmp_path):
                     "-o", exe, os.path.join(HERE, "fp64_sqrt_check.cu")], check=True)
     out = subprocess.run([exe], check=True, capture_output=True, text=True).stdout
     assert out.strip() == "differ 0", out
+
+
+def test_transposed_friction_takes_the_reciprocal_depth(tmp_path):
+    """The depth part of the transposed friction holds 1 / h to an ulp
+    (tests/fp64_vjp_check.cu): within two units in the last place."""
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    exe = str(tmp_path / "fp64_vjp_check")
+    subprocess.run([nvcc, "-O3", "-std=c++17", "-gencode", "arch=compute_103a,code=sm_103a",
+                    "-o", exe, os.path.join(HERE, "fp64_vjp_check.cu")], check=True)
+    out = subprocess.run([exe], check=True, capture_output=True, text=True).stdout
+    assert int(out.split()[1]) <= 2, out
