@@ -206,3 +206,14 @@ def test_early_halo_schedule_is_bitwise_equal(precision, tile, cpt):
     for other in runs[1:]:
         for a, b in zip(runs[0], other):
             assert np.array_equal(a, b)
+
+
+def test_autotuner_does_not_slow_a_mesh_that_stays_on_chip(tmp_path, monkeypatch):
+    """10,082 FP32 cells: no tile shape comes near the on-chip step (a factor
+    of four between them), so the answer is the library's own choice."""
+    pytest.importorskip("torch")
+    from paper_1807_00672_gb300 import autotune
+    ensure_built()
+    monkeypatch.setenv("SWE_TUNE_CACHE", str(tmp_path / "tune.json"))
+    r = autotune.tune([inputs.water_drop_case(n=71)], "f32")
+    assert (r["tile"], r["cells_per_thread"], r["stages"], r["halo_schedule"]) == (0, 0, 0, 0)
