@@ -612,28 +612,20 @@ int build_host_mesh(const double* xy, int64_t V, const int32_t* tri_in, int64_t 
   return 0;
 }
 
-bool build_resident_parts(const HostMesh& m, const double* xy, const int32_t* tri, bool is_morton,
-                          int32_t nparts, ResidentParts& out) {
+static bool cut_parts(const HostMesh& m, const double* xy, const int32_t* tri, bool is_morton,
+                      int32_t nparts, ResidentParts& out) {
   const int64_t T = m.T;
   const HostEdges& ed = m.edges;
   out = ResidentParts();
   if (nparts < 1 || nparts > T || (int64_t)ed.of_half.size() != 3 * T) return false;
-  // Host threads over the parts (ranges whose thread cannot start run here).
+  // Host threads over the parts.
   const unsigned nth = (unsigned)std::min<int64_t>(
       std::min(8u, std::max(1u, std::thread::hardware_concurrency())), std::min<int64_t>(nparts, T / 4000 + 1));
   auto over_parts = [&](auto&& body) {
-    std::vector<std::thread> pool;
-    unsigned started = 0;
-    auto run = [&](unsigned k) {
-      body((int32_t)((int64_t)nparts * k / nth), (int32_t)((int64_t)nparts * (k + 1) / nth));
-    };
-    try {
-      for (; started + 1 < nth; ++started) pool.emplace_back(run, started + 1);
-    } catch (...) {
-    }
-    run(0);
-    for (unsigned k = started + 1; k < nth; ++k) run(k);
-    for (std::thread& th : pool) th.join();
+    if (!on_threads(nth, [&](unsigned k) {
+          body((int32_t)((int64_t)nparts * k / nth), (int32_t)((int64_t)nparts * (k + 1) / nth));
+        }))
+      throw std::bad_alloc();
   };
   // internal cells in Morton order, and the part of each
   std::vector<int32_t> ord, part(T), local(T), nshared(nparts, 0);
@@ -771,6 +763,15 @@ bool build_resident_parts(const HostMesh& m, const double* xy, const int32_t* tr
   });
   // index 0x3fff of face 3 would read as a wall
   return out.cell_cap < 0x3fff && out.halo_cap < 0x3fff;
+}
+
+bool build_resident_parts(const HostMesh& m, const double* xy, const int32_t* tri, bool is_morton,
+                          int32_t nparts, ResidentParts& out) noexcept {
+  try {
+    return cut_parts(m, xy, tri, is_morton, nparts, out);
+  } catch (...) {
+    return false;
+  }
 }
 
 }  // namespace swe

@@ -2,8 +2,10 @@
 // locality renumbering and per-tile face lists. No CUDA in here.
 #pragma once
 
+#include <atomic>
 #include <cstdint>
 #include <new>
+#include <thread>
 #include <vector>
 
 namespace swe {
@@ -20,6 +22,32 @@ int guarded(F&& body) noexcept {
   } catch (...) {
     return -1;
   }
+}
+
+// Runs body(k) for k = 0 .. n - 1, on host threads where they start and else on
+// the calling one. No exception leaves a thread, nor this call before every
+// thread has ended: false if a body threw.
+template <typename F>
+bool on_threads(unsigned n, F&& body) noexcept {
+  std::atomic<bool> ok{true};
+  auto one = [&](unsigned k) noexcept {
+    try {
+      body(k);
+    } catch (...) {
+      ok = false;
+    }
+  };
+  std::vector<std::thread> pool;
+  unsigned started = 1;
+  try {
+    pool.reserve(n);
+    for (; started < n; ++started) pool.emplace_back(one, started);
+  } catch (...) {
+  }
+  one(0);
+  for (unsigned k = started; k < n; ++k) one(k);
+  for (std::thread& t : pool) t.join();
+  return ok;
 }
 
 // Encoding of one side of a tile face record:
@@ -115,8 +143,9 @@ void order_records_for_banks(HostMesh& m);
 
 // Cuts a mesh built with keep_edges into nparts parts of nearly equal size,
 // consecutive in the Morton order of the centroids (whatever order the mesh
-// has). Returns false if a part does not fit the record's 14-bit indices.
+// has). Returns false if a part does not fit the record's 14-bit indices or
+// there is no host memory.
 bool build_resident_parts(const HostMesh& m, const double* xy, const int32_t* tri, bool is_morton,
-                          int32_t nparts, ResidentParts& out);
+                          int32_t nparts, ResidentParts& out) noexcept;
 
 }  // namespace swe
