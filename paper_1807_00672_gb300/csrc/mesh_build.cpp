@@ -299,20 +299,9 @@ void order_records_for_banks(HostMesh& m) {
       std::copy(l.begin(), l.end(), m.tlen.begin() + r0);
     }
   };
-  if (nth == 1) {
-    work(0, nt);
-    return;
-  }
-  // Ranges whose thread cannot be started are done on this thread.
-  std::vector<std::thread> pool;
-  unsigned started = 0;
-  try {
-    for (; started < nth; ++started)
-      pool.emplace_back(work, nt * started / nth, nt * (started + 1) / nth);
-  } catch (...) {
-  }
-  for (unsigned k = started; k < nth; ++k) work(nt * k / nth, nt * (k + 1) / nth);
-  for (std::thread& th : pool) th.join();
+  // A tile is reordered whole or not at all: where memory runs out, the rest
+  // keep their order.
+  on_threads(nth, [&](unsigned k) { work(nt * k / nth, nt * (k + 1) / nth); });
 }
 
 int build_host_mesh(const double* xy, int64_t V, const int32_t* tri_in, int64_t T, int order,

@@ -138,7 +138,8 @@ int build_host_mesh(const double* xy, int64_t V, const int32_t* tri, int64_t T, 
                     bool keep_edges = false);
 
 // The bank order of build_host_mesh's bank_order, applied afterwards to every
-// tile (host threads over tiles).
+// tile (host threads over tiles); without host memory the records keep their
+// order.
 void order_records_for_banks(HostMesh& m);
 
 // Cuts a mesh built with keep_edges into nparts parts of nearly equal size,

@@ -27,3 +27,9 @@ def test_parts_are_left_out(checker):
     r = subprocess.run([checker, "parts"], capture_output=True, text=True)
     assert r.returncode == 0 and r.stdout.startswith("ok "), (r.returncode, r.stdout, r.stderr)
     assert int(r.stdout.split()[1]) > 30
+
+
+def test_records_keep_their_order(checker):
+    r = subprocess.run([checker, "banks"], capture_output=True, text=True)
+    assert r.returncode == 0 and r.stdout.startswith("ok "), (r.returncode, r.stdout, r.stderr)
+    assert int(r.stdout.split()[1]) > 3
