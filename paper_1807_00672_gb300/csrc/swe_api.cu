@@ -788,26 +788,19 @@ swe_status create_batch(int32_t n, const double* const* xy, const int64_t* n_nod
   std::vector<int> rc(n, 0);
   auto over_scenarios = [&](auto&& body) {  // on parallel host threads
     const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
-    const int nthr = (int)std::min<unsigned>((unsigned)n, std::min(16u, hw));
     std::atomic<int> next{0};
-    auto work = [&]() {
+    return swe::on_threads(std::min((unsigned)n, std::min(16u, hw)), [&](unsigned) {
       for (int i = next++; i < n; i = next++) body(i);
-    };
-    std::vector<std::thread> pool;
-    try {  // the calling thread takes every scenario no worker takes
-      for (int k = 1; k < nthr; ++k) pool.emplace_back(work);
-    } catch (...) {
-    }
-    work();
-    for (auto& t : pool) t.join();
+    });
   };
-  over_scenarios([&](int i) {
-    rc[i] = swe::build_host_mesh(xy[i], n_nodes[i], tri[i], n_tris[i], p.order,
-                                 kernel == SWE_KERNEL_TILED ? tile : 0, kernel == SWE_KERNEL_EDGE,
-                                 hm[i],
-                                 kernel == SWE_KERNEL_TILED && p.precision == SWE_F32 && !keep_edges,
-                                 keep_edges);
-  });
+  if (!over_scenarios([&](int i) {
+        rc[i] = swe::build_host_mesh(xy[i], n_nodes[i], tri[i], n_tris[i], p.order,
+                                     kernel == SWE_KERNEL_TILED ? tile : 0, kernel == SWE_KERNEL_EDGE,
+                                     hm[i],
+                                     kernel == SWE_KERNEL_TILED && p.precision == SWE_F32 && !keep_edges,
+                                     keep_edges);
+      }))
+    return SWE_ENOMEM;
   for (int i = 0; i < n; ++i) {
     if (rc[i] == -2) return SWE_EMESH;
     if (rc[i] != 0) return SWE_EINVAL;
@@ -928,12 +921,7 @@ swe_status create_batch(int32_t n, const double* const* xy, const int64_t* n_nod
   // The bank order of the FP32 tiles was left out where the resident kernel
   // might step the mesh.
   if (keep_edges && m->res.nblocks == 0 && kernel == SWE_KERNEL_TILED && p.precision == SWE_F32)
-    over_scenarios([&](int i) {
-      try {
-        swe::order_records_for_banks(hm[i]);
-      } catch (...) {  // no host memory: the records stay in their order, same results
-      }
-    });
+    over_scenarios([&](int i) { swe::order_records_for_banks(hm[i]); });
 
   // Device layout.
   const int64_t T = m->T, Tp = m->Tp, E = m->E, R = recs, H = halos;

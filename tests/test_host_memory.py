@@ -33,3 +33,21 @@ def test_records_keep_their_order(checker):
     r = subprocess.run([checker, "banks"], capture_output=True, text=True)
     assert r.returncode == 0 and r.stdout.startswith("ok "), (r.returncode, r.stdout, r.stderr)
     assert int(r.stdout.split()[1]) > 3
+
+
+
+def test_a_batch_without_memory_is_an_error(tmp_path):
+    """swe_mesh_create_batch, whose scenarios are built on several threads
+    (tests/batch_memory_check.cpp), in a process without a GPU."""
+    from paper_1807_00672_gb300 import build
+    cxx = shutil.which("g++")
+    if cxx is None:
+        pytest.skip("g++ not available")
+    lib = build.build()
+    out = str(tmp_path / "batch_memory_check")
+    subprocess.run([cxx, "-O2", "-std=c++17", "-pthread", "-o", out,
+                    os.path.join(HERE, "batch_memory_check.cpp"), lib,
+                    f"-Wl,-rpath,{os.path.dirname(lib)}", "-I", os.path.join(ROOT, "include")], check=True)
+    r = subprocess.run([out], capture_output=True, text=True, env=dict(os.environ, CUDA_VISIBLE_DEVICES=""))
+    assert r.returncode == 0 and r.stdout.startswith("ok "), (r.returncode, r.stdout, r.stderr)
+    assert int(r.stdout.split()[1]) > 10
