@@ -4,6 +4,7 @@
 
 #include <atomic>
 #include <cstdint>
+#include <exception>
 #include <new>
 #include <thread>
 #include <vector>
@@ -49,6 +50,19 @@ bool on_threads(unsigned n, F&& body) noexcept {
   for (std::thread& t : pool) t.join();
   return ok;
 }
+
+// Runs f if an exception (host memory) passes the scope it stands in: a handle
+// under construction goes with it.
+template <typename F>
+struct OnThrow {
+  F f;
+  int before = std::uncaught_exceptions();
+  explicit OnThrow(F g) : f(g) {}
+  OnThrow(const OnThrow&) = delete;
+  ~OnThrow() {
+    if (std::uncaught_exceptions() > before) f();
+  }
+};
 
 // Encoding of one side of a tile face record:
 //   >= 0             tile + q for the cell of another tile at index q of the

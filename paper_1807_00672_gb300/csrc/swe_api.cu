@@ -812,6 +812,7 @@ swe_status create_batch(int32_t n, const double* const* xy, const int64_t* n_nod
   CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
 
   swe_mesh* m = new swe_mesh();
+  swe::OnThrow on_throw([m] { swe_mesh_destroy(m); });
   m->prm = p;
   m->device = dev;
   m->sms = sms;
@@ -1360,6 +1361,7 @@ swe_status state_init(swe_mesh* m, const double* h, const double* hu, const doub
   swe_state* s = new swe_state();
   s->mesh = m;
   retain_mesh(m);
+  swe::OnThrow on_throw([s] { swe_state_destroy(s); });
   const bool interleaved = (m->kernel == SWE_KERNEL_TILED);
   Layout L;
   if (interleaved) {

@@ -467,6 +467,7 @@ swe_status grad_record(swe_state* s, int64_t n_steps, int64_t checkpoint_every,
   swe_tape* t = new swe_tape();
   t->mesh = m;
   retain_mesh(m);
+  swe::OnThrow on_throw([t] { free_tape(t); });
   t->stream = m->stream;
   t->N = n_steps;
   t->K = std::min(checkpoint_every, n_steps);

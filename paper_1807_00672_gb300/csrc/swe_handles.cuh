@@ -218,11 +218,11 @@ void launch_forward(const swe_mesh* m, const swe::DevState<double>& ds, cudaStre
                     bool back = false);
 // Resident kernel (swe_resident.cu). The most cells one block can keep;
 // resident_build cuts a mesh whose host meshes kept their edges into parts
-// (m->res.nblocks stays 0 if they do not fit), resident_upload copies them
+// (m->res.nblocks stays 0 if they do not fit or host memory runs out), resident_upload copies them
 // into the mesh's arena; one launch of up to n steps.
 int64_t resident_max_cells(const swe_mesh* m);
 void resident_build(swe_mesh* m, const std::vector<swe::HostMesh>& hm, const double* const* xy,
-                    const int32_t* const* tri);
+                    const int32_t* const* tri) noexcept;
 swe_status resident_upload(swe_mesh* m);
 cudaError_t launch_resident(const swe_state* s, int64_t n, cudaStream_t st);
 // Caller order (FP64) -> internal order in the mesh precision, and back;

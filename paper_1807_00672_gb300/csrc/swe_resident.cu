@@ -102,10 +102,9 @@ int64_t resident_max_cells(const swe_mesh* m) {
   return c;
 }
 
-void resident_build(swe_mesh* m, const std::vector<swe::HostMesh>& hm, const double* const* xy,
-                    const int32_t* const* tri) {
+static void build(swe_mesh* m, const std::vector<swe::HostMesh>& hm, const double* const* xy,
+                  const int32_t* const* tri) {
   ResidentMesh& r = m->res;
-  r = ResidentMesh();
   int coop = 0;
   if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, m->device) != cudaSuccess || !coop) {
     cudaGetLastError();
@@ -223,6 +222,16 @@ void resident_build(swe_mesh* m, const std::vector<swe::HostMesh>& hm, const dou
   }
   r.npub = (int32_t)npub;
   r.nblocks = (int32_t)blocks.size();
+}
+
+void resident_build(swe_mesh* m, const std::vector<swe::HostMesh>& hm, const double* const* xy,
+                    const int32_t* const* tri) noexcept {
+  m->res = ResidentMesh();
+  try {
+    build(m, hm, xy, tri);
+  } catch (...) {  // no host memory: the mesh steps without its parts
+    m->res = ResidentMesh();
+  }
 }
 
 swe_status resident_upload(swe_mesh* m) {

@@ -2,9 +2,9 @@
 // operator new failing from the k-th allocation on, on whichever host thread
 // that falls, for many k up to the number a build needs, each stage returns
 // (or throws std::bad_alloc on the calling thread) with every thread joined,
-// and works again afterwards. argv[1]: "parts" (build_resident_parts: false)
-// or "banks" (order_records_for_banks: each tile reordered or left alone).
-// Prints "ok <failures seen>" or the first difference. Test code: built and
+// and works again afterwards. argv[1]: "parts" (build_resident_parts: false),
+// "banks" (order_records_for_banks: each tile reordered or left alone) or
+// "guard" (OnThrow, which gives up handles under construction). Prints "ok <failures seen>" or the first difference. Test code: built and
 // run by tests/test_host_memory.py.
 #include <atomic>
 #include <cstdio>
@@ -28,7 +28,30 @@ void* operator new(std::size_t n) {
 void operator delete(void* p) noexcept { std::free(p); }
 void operator delete(void* p, std::size_t) noexcept { std::free(p); }
 
+// OnThrow: runs on the way of an exception out of its scope, also one thrown
+// while another is under way, and not on a return.
+static int g_ran = 0;
+static void scope(bool throws) {
+  swe::OnThrow on_throw([] { ++g_ran; });
+  if (throws) throw std::bad_alloc();
+}
+struct Unwinding {
+  ~Unwinding() { scope(false); }
+};
+static int guard_check() {
+  scope(false);
+  if (g_ran != 0) return 1;
+  try {
+    Unwinding u;
+    scope(true);
+  } catch (const std::bad_alloc&) {
+  }
+  std::printf("ok %d\n", g_ran);
+  return g_ran == 1 ? 0 : 1;
+}
+
 int main(int, char** argv) {
+  if (!std::strcmp(argv[1], "guard")) return guard_check();
   const bool banks = !std::strcmp(argv[1], "banks");
   const int32_t nx = banks ? 420 : 120, ny = banks ? 250 : 100;  // threads from 200,000 and 4,000 cells
   std::vector<double> xy;

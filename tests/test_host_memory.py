@@ -36,6 +36,11 @@ def test_records_keep_their_order(checker):
 
 
 
+def test_a_handle_under_construction_goes_with_the_exception(checker):
+    r = subprocess.run([checker, "guard"], capture_output=True, text=True)
+    assert r.returncode == 0 and r.stdout.strip() == "ok 1", (r.returncode, r.stdout, r.stderr)
+
+
 def test_a_batch_without_memory_is_an_error(tmp_path):
     """swe_mesh_create_batch, whose scenarios are built on several threads
     (tests/batch_memory_check.cpp), in a process without a GPU."""
