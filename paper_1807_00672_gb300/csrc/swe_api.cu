@@ -1536,6 +1536,13 @@ swe_status swe_advance(swe_state* s, double t_end, int64_t* n_steps) {
   set_end(s, t_end);
   s->open_ended = false;
   CK(cudaGetLastError());
+  bool ahead = false;  // else there is nothing to queue
+  for (int i = 0; i < nscen(s->mesh); ++i)
+    ahead = ahead || (!s->host_ctl[i].err && s->host_ctl[i].t < t_end);
+  if (!ahead) {
+    if (n_steps) *n_steps = 0;
+    return status_all(s);
+  }
   do {  // launches that find the end time reached take no step
     st = queue_steps(s, s->mesh->res.nblocks > 0 ? kStepsPerResident : kStepsPerGraph);
     if (st != SWE_OK) return st;

@@ -108,3 +108,30 @@ def test_a_rate_that_overflows_is_an_error(kernel, prec):
             call(st)
         assert ei.value.status == swe.SWE_ENAN
         assert st.info()["err"] == 1
+
+
+@pytest.mark.parametrize("kernel", ["tiled", "edge", "auto"])
+def test_advance_to_a_time_already_reached(kernel):
+    """No step, the state as it was, and later steps as if nothing had been
+    asked; with an error latched, that error."""
+    ensure_built()
+    case = inputs.random_flow_case(nx=37, ny=23, seed=41)
+    mesh = swe.Mesh(case.mesh.xy, case.mesh.tri, precision="f64", kernel=kernel)
+    a, b = (swe.State(mesh, case.h, case.hu, case.hv, case.z, case.n) for _ in range(2))
+    for st in (a, b):
+        st.run(10)
+    t = a.t
+    for end in (t, 0.5 * t, 0.0, -1.0, -np.inf):
+        assert a.advance(end) == 0 and a.t == t and a.info()["steps"] == 10
+    for st in (a, b):
+        st.run(5)
+        assert st.advance(1.5 * t) > 0 and st.t == 1.5 * t
+    for x, y in zip(a.fields(), b.fields()):
+        assert np.array_equal(x, y)
+    case.hu[100] = 1e200
+    case.n[:] = 0.0
+    st = swe.State(mesh, case.h, case.hu, case.hv, case.z, case.n)
+    for end in (1e3, 0.0, 1e3):
+        with pytest.raises(swe.SweError) as ei:
+            st.advance(end)
+        assert ei.value.status == swe.SWE_ENAN
