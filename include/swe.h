@@ -28,6 +28,11 @@
  *   - Handles are owned by the caller and freed with the matching destroy.
  *     Destroying a mesh that states still use is allowed: the mesh is freed
  *     when the last of them is destroyed. Handles are not thread-safe.
+ *   - Device memory of destroyed states and tapes is kept for the next ones
+ *     of the process, at most 2 GiB per device and in pieces above 64 MiB only
+ *     where half of the device was free. It is given back when the last mesh
+ *     of the process is destroyed, or when an allocation of this library fails
+ *     without it.
  */
 #ifndef SWE_H
 #define SWE_H
@@ -46,7 +51,7 @@ typedef int swe_status;
                                an edge shared by more than two triangles, empty mesh */
 #define SWE_ENOMEM (-3)     /* device or host allocation failed */
 #define SWE_ECUDA (-4)      /* a CUDA runtime call failed (no device, launch error) */
-#define SWE_ENAN (-5)       /* a non-finite value appeared in the state */
+#define SWE_ENAN (-5)       /* a non-finite value appeared in the state or in its CFL rate */
 #define SWE_ETIMEOUT (-7)   /* a bounded device-side wait ran out */
 #define SWE_EDRY (-8)       /* no wet cell left: the CFL time step is undefined */
 #define SWE_ESTATE (-9)     /* call not valid for this handle (e.g. wrong precision) */
@@ -68,8 +73,13 @@ typedef enum {
 /* Kernel structure of one step. */
 typedef enum {
   SWE_KERNEL_AUTO = 0,  /* SWE_KERNEL_TILED; SWE_KERNEL_EDGE for a single mesh in
-                           SWE_ORDER_RCM, whose tiles would be thin strips; small meshes
-                           stay on chip for many steps (see swe_params.tile) */
+                           SWE_ORDER_RCM, whose tiles would be thin strips. A mesh or
+                           ensemble that fits (about 330,000 FP32 or 180,000 FP64 cells,
+                           no more scenarios than SMs) stays on chip for the steps of a
+                           call, if its shape is left to the library: tile, stages,
+                           cells_per_thread and halo_schedule all 0. The results are
+                           SWE_KERNEL_TILED's, bit for bit, in SWE_ORDER_RCM too; gradients
+                           are recorded with SWE_KERNEL_TILED's step */
   SWE_KERNEL_EDGE = 1,  /* two launches: per-edge fluxes to HBM, then a per-cell gather
                            and update (the paper's two parallel loops, Sec. 2.3) */
   SWE_KERNEL_TILED = 2  /* one launch: each block stages a tile of cells in shared
@@ -87,7 +97,10 @@ typedef struct {
   int32_t kernel;     /* swe_kernel (default SWE_KERNEL_AUTO) */
   int32_t tile;       /* cells per tile of SWE_KERNEL_TILED; tile / cells_per_thread threads
                          per block must be 32, 64, 128 or 256; 0 = default (512 in
-                         FP32 at 2 cells per thread, else 256) */
+                         FP32 at 2 cells per thread, else 256; 256 in FP32 too for up to
+                         6,000,000 cells in all where stages, cells_per_thread and
+                         halo_schedule are 0 as well and no cell is a ghost). A value
+                         other than 0 keeps the mesh off the chip (see SWE_KERNEL_AUTO) */
   int32_t stages;     /* shared-memory pipeline stages of SWE_KERNEL_TILED (2 or 3);
                          0 = default (2) */
   int32_t cells_per_thread;  /* cells each thread updates per tile (1 or 2); 0 = default (2) */
@@ -493,7 +506,8 @@ swe_status swe_state_halo_unpack(swe_state* state, const int32_t* cells, int64_t
                                  const double* buf);
 
 /* Queues a copy of the CFL time step of the current state (Sec. 2.2,
- * Courant 0.7, over its non-ghost cells) to the DEVICE double *dt.
+ * Courant 0.7, over its non-ghost cells; +inf if none of them is wet) to the
+ * DEVICE double *dt.
  * Single-scenario meshes. No synchronisation. */
 swe_status swe_state_dt_device(const swe_state* state, double* dt);
 

@@ -287,7 +287,8 @@ constexpr int kSmallTileF32 = 256;
 constexpr int64_t kSmallTileCells = 6000000;
 constexpr int kDefaultTileF64 = 256;
 // No mesh above this many cells fits the resident kernel (the chip's shared
-// memory holds about 330,000 FP32 or 175,000 FP64 cells).
+// memory holds about 330,000 FP32, 320,000 with the depth residual, or 180,000
+// FP64 cells).
 constexpr int64_t kResidentCellsF32 = 340000, kResidentCellsF64 = 180000;
 // Several scenarios: up to kEnsembleWaves waves of work chunks, of at least
 // kWaveTiles tiles each. More waves balance uneven scenarios better, but each
@@ -920,7 +921,11 @@ swe_status create_batch(int32_t n, const double* const* xy, const int64_t* n_nod
 
   if (keep_edges && m->T <= (int64_t)sms * resident_max_cells(m)) resident_build(m, hm, xy, tri);
   // The bank order of the FP32 tiles was left out where the resident kernel
-  // might step the mesh.
+  // might step the mesh: it takes 7 ms of host time at 10,000 cells and 85 at
+  // 105,000 (one thread below 200,000), and what still runs the tiles of a
+  // resident mesh, recordings and adjoints of gradients, gains 0.1 to 3 % from
+  // it (40 recorded steps 0.344 ms without and 0.342 with it at 10,000 cells,
+  // 0.454 and 0.452 at 105,000, 0.529 and 0.515 at 320,000).
   if (keep_edges && m->res.nblocks == 0 && kernel == SWE_KERNEL_TILED && p.precision == SWE_F32)
     over_scenarios([&](int i) { swe::order_records_for_banks(hm[i]); });
 
