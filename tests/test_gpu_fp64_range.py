@@ -46,3 +46,13 @@ def test_transposed_friction_takes_the_reciprocal_depth(tmp_path):
                     "-o", exe, os.path.join(HERE, "fp64_vjp_check.cu")], check=True)
     out = subprocess.run([exe], check=True, capture_output=True, text=True).stdout
     assert int(out.split()[1]) <= 2, out
+
+
+def test_the_time_step_is_the_ieee_quotient(tmp_path):
+    """courant / rate, bit for bit (tests/fp64_dt_check.cu)."""
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    exe = str(tmp_path / "fp64_dt_check")
+    subprocess.run([nvcc, "-O3", "-std=c++17", "-gencode", "arch=compute_103a,code=sm_103a",
+                    "-o", exe, os.path.join(HERE, "fp64_dt_check.cu")], check=True)
+    out = subprocess.run([exe], check=True, capture_output=True, text=True).stdout
+    assert out.strip() == "differ 0", out
