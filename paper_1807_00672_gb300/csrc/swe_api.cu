@@ -926,8 +926,11 @@ swe_status create_batch(int32_t n, const double* const* xy, const int64_t* n_nod
   // resident mesh, recordings and adjoints of gradients, gains 0.1 to 3 % from
   // it (40 recorded steps 0.344 ms without and 0.342 with it at 10,000 cells,
   // 0.454 and 0.452 at 105,000, 0.529 and 0.515 at 320,000).
-  if (keep_edges && m->res.nblocks == 0 && kernel == SWE_KERNEL_TILED && p.precision == SWE_F32)
-    over_scenarios([&](int i) { swe::order_records_for_banks(hm[i]); });
+  auto order_if_tiled = [&] {
+    if (keep_edges && m->res.nblocks == 0 && kernel == SWE_KERNEL_TILED && p.precision == SWE_F32)
+      over_scenarios([&](int i) { swe::order_records_for_banks(hm[i]); });
+  };
+  order_if_tiled();
 
   // Device layout.
   const int64_t T = m->T, Tp = m->Tp, E = m->E, R = recs, H = halos;
@@ -964,6 +967,7 @@ swe_status create_batch(int32_t n, const double* const* xy, const int64_t* n_nod
   if (got != cudaSuccess && m->res.nblocks > 0) {  // without the resident kernel's parts
     cudaGetLastError();
     m->res = ResidentMesh();
+    order_if_tiled();
     L.total = bare;
     got = device_alloc(&m->arena.base, L.total);
   }
